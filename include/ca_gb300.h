@@ -95,6 +95,7 @@ typedef struct {
 
 #define CA_STATUS_NONFINITE 1
 #define CA_STATUS_SOLVE_TIMEOUT 16 /* dev_info[1] of calu_gesv_mixed: a solve gave up waiting */
+#define CA_STATUS_PANEL_TIMEOUT 64 /* dev_info[1]: a panel node gave up waiting for its cluster     */
 #define CA_STATUS_REFACTORED 32    /* dev_info[1] of calu_gesv_mixed: the fallback refactorization ran */
 
 /* Correction method of calu_gesv_mixed's refinement */

@@ -1,6 +1,7 @@
 // panel_lu.cu -- TSLU tournament pivoting and the LU panel steps of CALU.
 //
-// Tree node = one thread-block cluster of G CTAs (G = 1, 2, 4, 8).  The node's
+// Nodes that fit the registers of a cluster run in panel_lu_reg.cu; the node
+// kernel here takes the larger ones.  Tree node = one thread-block cluster of G CTAs (G = 1, 2, 4, 8).  The node's
 // rows (a leaf of the panel, or the stacked candidate rows of its children)
 // are split in contiguous chunks over the G CTAs' shared memory; GEPP runs on
 // the distributed tile: per column, a warp-shuffle argmax inside each CTA,
@@ -13,34 +14,13 @@
 
 #include "ca_internal.cuh"
 #include "device_once.cuh"
+#include "lu_node.cuh"
 
 namespace cagb {
 
 constexpr int kNodeThreads = 256;
 constexpr int kNodeWarps = kNodeThreads / 32;
 constexpr size_t kNodeSmemBudget = 220 * 1024;
-
-struct TsluNodeArgs {
-  const double *P;  // panel (row 0 = first row of the panel), ld lda
-  int lda, mk, bk;
-  int leaf_rows;
-  int is_leaf;      // nodes of this launch are the leaves
-  int is_root;      // the single node of this launch is the root
-  RoundDesc rd;     // merge round (when !is_leaf)
-  const int *cand_in;
-  const int *ncand_in;
-  int *cand_out;
-  int *ncand_out;
-  int cand_ld;      // ints per node in the candidate buffers (= b)
-  int rloc;         // tile rows per CTA
-  // root outputs
-  double *lu11;     // bk x bk, ld cand_ld
-  int *perm_src, *perm_dst, *perm_cnt;
-  int *ipiv_k;      // ipiv + kb
-  int ipiv_base;    // kb
-  const int *skip;  // nonzero: a stage enqueued ahead that is not needed, do nothing
-  int *dev_info;    // [0] info, [1] status
-};
 
 struct TsluSmem {
   // layout inside dynamic shared memory
@@ -400,66 +380,14 @@ __global__ void __launch_bounds__(kNodeThreads, 1) tslu_node_kernel(TsluNodeArgs
     node_sync(cl, G);  // keep shared memory alive until rank 0 has read it
     return;
   }
-  int *sel = s.work;            // bk selected labels
-  int *rev_top = s.work + bk;   // position of top label x (>= 0) or -(slot+1)
-  int *top_c = s.work + 2 * bk; // label at top position t
-  int *far_c = s.work + 3 * bk; // label at far position sel[s] (sel[s] >= bk)
+  int *sel = s.work;  // bk chosen labels
   for (int t = tid; t < bk; t += kNodeThreads) {
     int q = t / rloc, l = t - q * rloc;
     sel[t] = (q == 0) ? s.lab[l] : *cl.map_shared_rank(s.lab + l, q);
   }
   __syncthreads();
   node_sync(cl, G);
-  if (tid == 0) {
-    for (int t = 0; t < bk; ++t) {
-      rev_top[t] = t;
-      top_c[t] = t;
-      far_c[t] = sel[t];
-    }
-    // LAPACK swap sequence: at step i, swap position i with the current
-    // position of the i-th selected row.
-    for (int i = 0; i < bk; ++i) {
-      int L = sel[i], pp, fslot = -1;
-      if (L < bk) {
-        int r = rev_top[L];
-        if (r >= 0) {
-          pp = r;
-        } else {
-          fslot = -r - 1;
-          pp = sel[fslot];
-        }
-      } else {
-        pp = L;
-        fslot = i;
-      }
-      a.ipiv_k[i] = a.ipiv_base + pp + 1;
-      if (pp == i) continue;
-      int Ci = top_c[i];
-      top_c[i] = L;
-      if (pp < bk) {
-        top_c[pp] = Ci;
-        rev_top[Ci] = pp;
-      } else {
-        far_c[fslot] = Ci;
-        rev_top[Ci] = -(fslot + 1);
-      }
-      if (L < bk) rev_top[L] = i;
-    }
-    int n = 0;
-    for (int t = 0; t < bk; ++t)
-      if (top_c[t] != t) {
-        a.perm_dst[n] = t;
-        a.perm_src[n] = top_c[t];
-        ++n;
-      }
-    for (int t = 0; t < bk; ++t)
-      if (sel[t] >= bk) {
-        a.perm_dst[n] = sel[t];
-        a.perm_src[n] = far_c[t];
-        ++n;
-      }
-    *a.perm_cnt = n;
-  }
+  if (tid < 32) lu_root_swaps(a, sel, s.work + bk);
 }
 
 // ---------------------------------------------------------------------------
@@ -618,6 +546,12 @@ static double gepp_flops(double r, double c) {
   return f;
 }
 
+static double node_flops(const TsluNodeArgs &args, int nodes) {
+  const double rows = args.is_leaf ? (args.leaf_rows < args.mk ? args.leaf_rows : args.mk)
+                                   : (double)args.rd.max_cnt * args.bk;
+  return nodes * gepp_flops(rows, args.bk);
+}
+
 static cudaError_t launch_tslu_node(const TsluNodeArgs &args, int nodes, int G, cudaStream_t st) {
   static std::atomic<unsigned long long> init{0};
   cudaError_t e = once_per_device(init, [] {
@@ -626,9 +560,7 @@ static cudaError_t launch_tslu_node(const TsluNodeArgs &args, int nodes, int G, 
   });
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  const double rows = args.is_leaf ? (args.leaf_rows < args.mk ? args.leaf_rows : args.mk)
-                                   : (double)args.rd.max_cnt * args.bk;
-  ProfScope ps(kClsTsluNode, st, nodes * gepp_flops(rows, args.bk));
+  ProfScope ps(kClsTsluNode, st, node_flops(args, nodes));
   cfg.gridDim = dim3(nodes * G);
   cfg.blockDim = dim3(kNodeThreads);
   cfg.dynamicSmemBytes = tslu_smem_bytes(args.rloc, args.bk);
@@ -641,6 +573,19 @@ static cudaError_t launch_tslu_node(const TsluNodeArgs &args, int nodes, int G, 
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, tslu_node_kernel, args);
+}
+
+// One round of nodes of at most R rows: in registers where they fit (see
+// panel_lu_reg.cu), else in the shared memory of a cluster.
+static cudaError_t tslu_round(TsluNodeArgs &a, int nodes, int R, cudaStream_t st) {
+  int G = tslu_reg_cluster(R, a.bk, nodes, &a.rloc);
+  if (G > 0) {
+    ProfScope ps(kClsTsluNode, st, node_flops(a, nodes));
+    return launch_tslu_reg(a, nodes, G, st);
+  }
+  G = pick_cluster(R, a.bk, nodes, &a.rloc);
+  if (G < 0) return cudaErrorInvalidValue;
+  return launch_tslu_node(a, nodes, G, st);
 }
 
 cudaError_t tslu_panel(int mk, int bk, double *P, int lda, int leaf_rows, const Plan &plan,
@@ -663,33 +608,25 @@ cudaError_t tslu_panel(int mk, int bk, double *P, int lda, int leaf_rows, const 
   a.dev_info = dev_info;
   // leaves
   int R = leaf_rows < mk ? leaf_rows : mk;
-  int rloc;
-  int G = pick_cluster(R, bk, plan.nleaves, &rloc);
-  if (G < 0) return cudaErrorInvalidValue;
   a.is_leaf = 1;
   a.is_root = (plan.nrounds == 0);
-  a.rloc = rloc;
   a.cand_in = nullptr;
   a.ncand_in = nullptr;
   a.cand_out = ws.cand[0];
   a.ncand_out = ws.ncand[0];
-  cudaError_t e = launch_tslu_node(a, plan.nleaves, G, st);
+  cudaError_t e = tslu_round(a, plan.nleaves, R, st);
   if (e != cudaSuccess) return e;
   int buf = 0;
   for (int r = 0; r < plan.nrounds; ++r) {
     const RoundDesc &rd = plan.r[r];
-    int Rm = rd.max_cnt * bk;
-    G = pick_cluster(Rm, bk, rd.n_out, &rloc);
-    if (G < 0) return cudaErrorInvalidValue;
     a.is_leaf = 0;
     a.is_root = (r == plan.nrounds - 1);
     a.rd = rd;
-    a.rloc = rloc;
     a.cand_in = ws.cand[buf];
     a.ncand_in = ws.ncand[buf];
     a.cand_out = ws.cand[buf ^ 1];
     a.ncand_out = ws.ncand[buf ^ 1];
-    e = launch_tslu_node(a, rd.n_out, G, st);
+    e = tslu_round(a, rd.n_out, rd.max_cnt * bk, st);
     if (e != cudaSuccess) return e;
     buf ^= 1;
   }
