@@ -111,9 +111,12 @@ const char *ca_strerror(int code);
 /* Workspace queries (host only, no GPU work).                              */
 /* ------------------------------------------------------------------------ */
 
-/* Bytes of device workspace `work` needed by calu_factor / tslu for an
- * m x n matrix with panel width b and this tree.  Also returns CA_OK or an
- * argument error exactly as calu_factor would for the same shape. */
+/* Bytes of device workspace `work` of calu_factor / tslu for an m x n matrix
+ * with panel width b and this tree.  Also returns CA_OK or an argument error
+ * exactly as calu_factor would for the same shape.  The size includes room
+ * for the trailing update's operands (see calu_factor); calu_factor also
+ * accepts a workspace without it, down to this query's size for a single
+ * panel (n = b), and then updates on the FP64 pipe. */
 int ca_calu_workspace(int m, int n, int b, const ca_tree_t *tree, size_t *work_bytes);
 
 /* Bytes of the CAQR reflector store `qtree` (the T factors of every tree
@@ -143,7 +146,13 @@ int ca_getrs_workspace(int n, int nrhs, size_t *work_bytes);
  *      original values, children in order);
  *   2. the rows are swapped at left and right of the panel (full width);
  *   3. L21 = A21 U11^-1 and U12 = L11^-1 A12, with L11 U11 the root's factors;
- *   4. A22 -= L21 U12 (Schur complement).
+ *   4. A22 -= L21 U12 (Schur complement).  With the queried workspace this
+ *      product runs on the tensor cores from exact 8-bit digits of the FP64
+ *      operands (7 digits, exact sums, two roundings of A22): at least as
+ *      close to the exact product as FP64 multiply-adds.  Rows and columns
+ *      holding values that are not finite, or near the ends of the range, are
+ *      multiplied in FP64.  dev_info[1] gets a bit (2, 4 or 8) if a bounded
+ *      wait of that kernel gave up.
  * Output in LAPACK getrf layout: unit L strictly below the diagonal, U on and
  * above; ipiv[i] (1-based, device, min(m,n) ints) is the row swapped with
  * row i, applied in order i = 0, 1, ....  Arguments: 1 m, 2 n, 3 A, 4 lda,

@@ -76,6 +76,14 @@ int lu_shape(int m, int n, int b, const ca_tree_t *tree, int *nl_max) {
   return CA_OK;
 }
 
+// Workspace of the FP64 trailing updates on the tensor cores (0 for a single
+// panel, which has none).
+size_t lu_f64_ws_bytes(int m, int n, int b) {
+  const int K = m < n ? m : n;
+  if (K == 0 || b >= n || b >= m || !tc_f64_pays(m - b, n - b, b)) return 0;
+  return tc_f64_ws_bytes(m - b, n - b, b);
+}
+
 // CALU panel workspace: the tournament buffers, then (2D operator) the
 // operator's candidate buffers of every node of a round
 size_t lu_ws_bytes(int nl, int bw, const ca_tree_t *tree) {
@@ -148,7 +156,8 @@ Lookahead *lookahead_for(cudaStream_t user) {
 // trailing update runs in FP64 (tcws == nullptr) or on the tensor cores with
 // `slices` digits (reduced precision, exact = per-diagonal accumulators).
 int calu_run(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, int *ipiv, void *work, int nl,
-             void *tcws, int slices, int exact, int *dev_info, cudaStream_t stream, const int *skip = nullptr) {
+             void *tcws, int slices, int exact, int *dev_info, cudaStream_t stream, const int *skip = nullptr,
+             void *f64ws = nullptr) {
   if (cudaMemsetAsync(dev_info, 0, 2 * sizeof(int), stream) != cudaSuccess) return CA_ERR_LAUNCH;
   const int K = m < n ? m : n;
   if (K == 0) return CA_OK;
@@ -159,8 +168,16 @@ int calu_run(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, int
   const int L = tree->leaf_rows;
   Lookahead *la = (K > b) ? lookahead_for(stream) : nullptr;
   if (la && cudaEventRecord(la->ev_next, stream) != cudaSuccess) return CA_ERR_LAUNCH;
+  // the panel's first update on the tensor cores makes L21's digits
+  bool split_a = true;
   auto update = [&](int mrows, int ncols, int kdim, const double *L21, const double *U12, double *C) -> cudaError_t {
     if (mrows <= 0 || ncols <= 0) return cudaSuccess;
+    if (f64ws && tc_f64_pays(mrows, ncols, kdim)) {
+      const cudaError_t e = gemm_minus_f64_tc(mrows, ncols, kdim, L21, lda, U12, lda, C, lda, split_a, f64ws,
+                                              dev_info + 1, stream, skip);
+      split_a = false;
+      return e;
+    }
     if (tcws)
       return gemm_minus_tc(mrows, ncols, kdim, L21, lda, U12, lda, C, lda, slices, exact, tcws, dev_info + 1, stream,
                            skip);
@@ -168,6 +185,7 @@ int calu_run(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, int
   };
   for (int kb = 0; kb < K; kb += b) {
     NvtxRange range("calu panel");
+    split_a = true;
     const int bk = (K - kb < b) ? K - kb : b;
     const int mk = m - kb;
     Plan plan;
@@ -321,7 +339,7 @@ int ca_calu_workspace(int m, int n, int b, const ca_tree_t *tree, size_t *work_b
   int rc = lu_shape(m, n, b, tree, &nl);
   if (rc == -5 || rc == -6) rc = (rc == -5) ? -3 : -4;  // positions in this call
   if (rc != CA_OK) return rc;
-  *work_bytes = lu_ws_bytes(nl, b < kMaxB ? b : kMaxB, tree);
+  *work_bytes = align256(lu_ws_bytes(nl, b < kMaxB ? b : kMaxB, tree)) + lu_f64_ws_bytes(m, n, b);
   return CA_OK;
 }
 
@@ -371,7 +389,11 @@ int calu_factor(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, 
   if (!dev_info) return -10;
   const int bw = b < kMaxB ? b : kMaxB;
   if (K > 0 && (!work || lwork < lu_ws_bytes(nl, bw, tree))) return CA_ERR_WORKSPACE;
-  return calu_run(m, n, A, lda, b, tree, ipiv, work, nl, nullptr, 0, 0, dev_info, stream);
+  // the trailing updates run on the tensor cores when the workspace has room
+  // for their operands' digits (the query's size), else on the FP64 pipe
+  const size_t base = align256(lu_ws_bytes(nl, bw, tree)), more = lu_f64_ws_bytes(m, n, b);
+  void *f64ws = (more > 0 && lwork >= base + more) ? (char *)work + base : nullptr;
+  return calu_run(m, n, A, lda, b, tree, ipiv, work, nl, nullptr, 0, 0, dev_info, stream, nullptr, f64ws);
 }
 
 int tslu(int m, int n, double *A, int lda, const ca_tree_t *tree, int *ipiv, void *work,

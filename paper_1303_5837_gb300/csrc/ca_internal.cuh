@@ -307,6 +307,15 @@ struct TcGemm {
   double sign;
   int S, exact;
   const int *skip;      // as for the LU launchers (null: always run)
+  // full: the result stands in for an FP64 product.  Vectors whose digits
+  // cannot (a value that is not finite, or a largest magnitude near the ends
+  // of the range) are multiplied in FP64 by the epilogue.  kexp: A's column k
+  // is taken times 2^-kexp[k] and B's row k times 2^kexp[k] (exact; null: 0).
+  // reuse_a: A's digits of the previous call with this workspace, A and kexp
+  // are still in place.
+  int full;
+  const int *kexp;
+  int reuse_a;
 };
 cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st);
 size_t tc_gemm_ws_bytes_batched(int m, int n, int k, int S, int nbatch);
@@ -315,6 +324,14 @@ bool tc_gemm_supported(int k, int S, int exact);
 cudaError_t gemm_minus_tc(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C,
                           int ldc, int S, int exact, void *ws, int *status, cudaStream_t st,
                           const int *skip = nullptr);
+
+// The FP64 Schur update C -= A B (m x k, k x n, k <= 128) from 7 digits on the
+// tensor cores (gemm_tc.cu): ws of tc_f64_ws_bytes for the largest m, n.
+constexpr int kTcF64Slices = 7;
+size_t tc_f64_ws_bytes(int m, int n, int k);
+bool tc_f64_pays(int m, int n, int k);
+cudaError_t gemm_minus_f64_tc(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C,
+                              int ldc, bool first, void *ws, int *status, cudaStream_t st, const int *skip);
 
 // CAQR tree update on the tensor cores (update_tc.cu)
 size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, int S);

@@ -30,6 +30,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <climits>
+
 #include "ca_internal.cuh"
 #include "device_once.cuh"
 
@@ -261,7 +263,39 @@ struct TcArgs {
   int sign;            // C -= sign * A B, sign = +1 or -1
   int *status;
   const int *skip;     // nonzero: a stage enqueued ahead that is not needed, do nothing
+  int full;            // vectors marked kExOdd are multiplied in FP64 from A and B
+  TcOperand A, B;
 };
+
+// Exponent mark of a vector that has no digits (TcGemm::full).
+constexpr int kExOdd = 1 << 20;
+
+// Element (v, k) of item b of an operand, 0 outside its structure.
+__device__ __forceinline__ double operand_at(const TcOperand &o, const double *X, int v, int k) {
+  const int r = (o.trans ? k : v) + o.roff, q = o.trans ? v : k;
+  if (o.shape == 0 || (o.shape == 1 && r > q) || (o.shape == 2 && r <= q))
+    return X[(long long)v * o.sv + (long long)k * o.sk];
+  return (o.shape == 1 && r == q) ? 1.0 : 0.0;
+}
+__device__ __forceinline__ const double *operand_item(const TcOperand &o, int b) {
+  return o.X + (long long)b * o.sb + (o.off ? o.off[b] : 0);
+}
+__device__ __forceinline__ int operand_k(const TcOperand &o, int b, bool last) {
+  return o.K_item ? o.K_item[b] : (last ? o.K_last : o.K);
+}
+
+// c - sign sum_k A(i, k) B(k, j) as a chain of FP64 multiply-adds: the
+// elements whose row or column has no digits.
+__device__ __noinline__ double odd_element(const TcArgs &a, int item, int i, int j, double c) {
+  const bool last = item == a.nbatch - 1;
+  const int K = min(operand_k(a.A, item, last), operand_k(a.B, item, last));
+  const double *X = operand_item(a.A, item), *Y = operand_item(a.B, item);
+  for (int k = 0; k < K; ++k) {
+    const double x = operand_at(a.A, X, i, k);
+    c = fma(a.sign > 0 ? -x : x, operand_at(a.B, Y, j, k), c);
+  }
+  return c;
+}
 
 // Operand tiles for one K block: S boxes of A digits (128 x bk) then S boxes
 // of B digits (bn x bk).
@@ -430,7 +464,9 @@ __global__ void __launch_bounds__(256, 2)
         if (col >= nvv) continue;
         const int sc = er + ec[j] - 16;  // C -= sign 2^sc value
         double c = cv[j];
-        if (a.exact) {
+        if (a.full && sc > kExOdd / 2) {
+          c = odd_element(a, item, row, col, c);
+        } else if (a.exact) {
           // value = T_hi 2^(8 (4 - dmax)) ... written relative to diagonal dmax:
           // sum_D acc_D 2^(-8 D) = T_hi 2^(-32) + T_lo 2^(-48)
           c -= scaled_rn(a.sign > 0 ? thi[j] : -thi[j], sc - 32);
@@ -463,7 +499,7 @@ __global__ void __launch_bounds__(256, 2)
 // --------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int S, int vpad, int kpad, int exact,
                                                     __nv_bfloat16 *__restrict__ out, int *__restrict__ ex,
-                                                    const int *skip) {
+                                                    const int *skip, int full, const int *kexp, int ksign) {
   if (skip && *skip) return;
   const int lane = threadIdx.x & 31;
   const int v = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -471,25 +507,28 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
   if (v >= vpad) return;
   const bool last = b == nbatch - 1;
   const int nv = o.nv_item ? o.nv_item[b] : (last ? o.nv_last : o.nv);
-  const int K = o.K_item ? o.K_item[b] : (last ? o.K_last : o.K);
-  const double *X = o.X + (long long)b * o.sb + (o.off ? o.off[b] : 0);
+  const int K = operand_k(o, b, last);
+  const double *X = operand_item(o, b);
   constexpr int kPer = 8;  // K <= 256
   double x[kPer];
+  int sh[kPer];            // the element is taken times 2^sh
   unsigned long long mx = 0;
+  int me = INT_MIN;        // largest exponent field + sh of a nonzero element
+  unsigned odd = 0;
 #pragma unroll
   for (int t = 0; t < kPer; ++t) {
     const int k = lane + 32 * t;
     double val = 0.0;
-    if (v < nv && k < K) {
-      const int r = (o.trans ? k : v) + o.roff, q = o.trans ? v : k;
-      if (o.shape == 0 || (o.shape == 1 && r > q) || (o.shape == 2 && r <= q))
-        val = X[(long long)v * o.sv + (long long)k * o.sk];
-      else if (o.shape == 1 && r == q)
-        val = 1.0;
-    }
+    if (v < nv && k < K) val = operand_at(o, X, v, k);
     x[t] = val;
     const unsigned long long bits = absbits(val);
     mx = bits > mx ? bits : mx;
+    sh[t] = 0;
+    if (full) {
+      if (kexp && k < K) sh[t] = ksign * kexp[k];
+      if (bits != 0) me = max(me, (int)(bits >> 52) + sh[t]);
+      odd |= (bits >> 52) == 0x7ffull;
+    }
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -502,6 +541,18 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
     const int E = (int)(mx >> 52);
     e = (E == 0) ? -1021 : E - 1022;
   }
+  if (full) {
+    me = __reduce_max_sync(0xffffffffu, me);
+    odd = __reduce_or_sync(0xffffffffu, odd);
+    if (mx != 0) {
+      e = me - 1022;
+      if (odd || e < -900 || e > 1000) {  // no digits: FP64 in the epilogue
+        e = kExOdd;
+#pragma unroll
+        for (int t = 0; t < kPer; ++t) x[t] = 0.0;
+      }
+    }
+  }
   if (lane == 0) ex[(long long)b * vpad + v] = e;
 #pragma unroll
   for (int t = 0; t < kPer; ++t) {
@@ -509,7 +560,7 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
     if (k >= kpad) continue;
     // F = round(x 2^(8S - e)) = sum_s d_s 256^(S-1-s), balanced digits
     // d_s in [-128, 127] for s >= 1 and |d_0| <= 256, all integer arithmetic
-    long long F = fixed_point_digits(x[t], e, S);
+    long long F = fixed_point_digits(x[t], e - sh[t], S);
     int dg[8];
 #pragma unroll
     for (int s = 7; s >= 1; --s) {
@@ -662,20 +713,20 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
   char *p = (char *)(((uintptr_t)ws + 255) & ~(uintptr_t)255);
   __nv_bfloat16 *sa = (__nv_bfloat16 *)p;
   p += align256(nb * S * mp * kp * 2);
-  __nv_bfloat16 *sb = (__nv_bfloat16 *)p;
-  p += align256(nb * S * np * kp * 2);
   int *ea = (int *)p;
   p += align256(nb * mp * 4);
+  __nv_bfloat16 *sb = (__nv_bfloat16 *)p;
+  p += align256(nb * S * np * kp * 2);
   int *eb = (int *)p;
-  {
+  if (!g.reuse_a) {
     ProfScope ps(kClsSplit, st, 0.0);
     split_kernel<<<dim3((mp + 7) / 8, g.nbatch), 256, 0, st>>>(g.A, g.nbatch, S, mp, kp, exact, sa, ea,
-                                                                g.skip);
+                                                                g.skip, g.full, g.kexp, -1);
   }
   {
     ProfScope ps(kClsSplit, st, 0.0);
     split_kernel<<<dim3((np + 7) / 8, g.nbatch), 256, 0, st>>>(g.B, g.nbatch, S, np, kp, exact, sb, eb,
-                                                                g.skip);
+                                                                g.skip, g.full, g.kexp, 1);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -711,6 +762,9 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
   a.sign = g.sign > 0 ? 1 : -1;
   a.status = status;
   a.skip = g.skip;
+  a.full = g.full;
+  a.A = g.A;
+  a.B = g.B;
   const size_t smem = cfg.smem;
   static std::atomic<unsigned long long> init{0};
   e = once_per_device(init, [] {
@@ -727,8 +781,8 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t gemm_minus_tc(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C,
-                          int ldc, int S, int exact, void *ws, int *status, cudaStream_t st, const int *skip) {
+static TcGemm schur_gemm(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
+                         int S, int exact, const int *skip) {
   TcGemm g = {};
   g.skip = skip;
   g.A.X = A;  // rows of A: element (i, k) at A[i + k lda]
@@ -747,7 +801,70 @@ cudaError_t gemm_minus_tc(int m, int n, int k, const double *A, int lda, const d
   g.sign = 1.0;
   g.S = S;
   g.exact = exact;
-  return gemm_tc(g, ws, status, st);
+  return g;
+}
+
+cudaError_t gemm_minus_tc(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C,
+                          int ldc, int S, int exact, void *ws, int *status, cudaStream_t st, const int *skip) {
+  return gemm_tc(schur_gemm(m, n, k, A, lda, B, ldb, C, ldc, S, exact, skip), ws, status, st);
+}
+
+// --------------------------------------------------------------------------
+// The FP64 Schur update on the tensor cores.  Seven digits of 8 bits hold
+// every operand to 2^-57 of its vector's largest magnitude, the digit sums are
+// exact and C is rounded twice, so the result is closer to the exact product
+// than 128 FP64 multiply-adds, each of which rounds C: relative error 7e-17
+// against 3.8e-16 (256 x 256 x 128, N(0,1)), backward error of the whole CALU
+// 5.6e-15 against 1.2e-14 (n = 2048, N(0,1)).  What the digits keep is
+// relative to the largest magnitude of the row of A (column of B), so A's
+// columns are first brought to one scale and B's rows scaled back (powers of
+// two, column_exp_kernel): badly scaled rows of the matrix, which make the columns of L21 grow
+// from pivot to pivot while the rows of U12 shrink, then lose nothing.
+// CALU + solve of n = 10240, b = 128: 681 -> 186 ms (622 ms of FP64 GEMM
+// became 120 ms here, most of it beside the next panel's tournament).
+// --------------------------------------------------------------------------
+// kexp[k]: exponent of the largest finite magnitude of column k of A (0 for a
+// column without one); one CTA per column.
+__global__ void __launch_bounds__(256) column_exp_kernel(int m, const double *__restrict__ A, int lda, int *kexp,
+                                                         const int *skip) {
+  if (skip && *skip) return;
+  __shared__ int red[8];
+  const double *a = A + (size_t)blockIdx.x * lda;
+  int E = 0;
+  for (int i = threadIdx.x; i < m; i += 256) {
+    const int e = (int)(absbits(a[i]) >> 52);
+    E = max(E, e == 0x7ff ? 0 : e);
+  }
+  E = __reduce_max_sync(0xffffffffu, E);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = E;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 0; w < 8; ++w) E = max(E, red[w]);
+    kexp[blockIdx.x] = E == 0 ? 0 : E - 1023;
+  }
+}
+
+size_t tc_f64_ws_bytes(int m, int n, int k) { return align256((size_t)k * 4) + 256 + tc_gemm_ws_bytes(m, n, k, kTcF64Slices); }
+
+// One 128 x 64 tile of digits costs about 15 us however little of it is used
+// (three launches, 28 products); the FP64 kernel as much at 64 x 64 x 64.
+// CALU of n = 600, b = 64 takes 4.25 ms with the line at 64 rows and columns,
+// 4.45 with it at 128, and of n = 1024 7.9 against 8.2.
+bool tc_f64_pays(int m, int n, int k) { return k >= 16 && k <= 128 && m >= 64 && n >= 64; }
+
+cudaError_t gemm_minus_f64_tc(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C,
+                              int ldc, bool first, void *ws, int *status, cudaStream_t st, const int *skip) {
+  char *p = (char *)(((uintptr_t)ws + 255) & ~(uintptr_t)255);
+  int *kexp = (int *)p;
+  TcGemm g = schur_gemm(m, n, k, A, lda, B, ldb, C, ldc, kTcF64Slices, 1, skip);
+  g.full = 1;
+  g.kexp = kexp;
+  g.reuse_a = !first;
+  if (first) {
+    ProfScope ps(kClsSplit, st, 0.0);
+    column_exp_kernel<<<k, 256, 0, st>>>(m, A, lda, kexp, skip);
+  }
+  return gemm_tc(g, p + align256((size_t)k * 4), status, st);
 }
 
 }  // namespace cagb
