@@ -121,7 +121,10 @@ int ca_calu_workspace(int m, int n, int b, const ca_tree_t *tree, size_t *work_b
 
 /* Bytes of the CAQR reflector store `qtree` (the T factors of every tree
  * node, see caqr_factor) and of the scratch workspace `work` for an m x n
- * matrix (m >= n) with panel width b. */
+ * matrix (m >= n) with panel width b.  As for calu_factor, work_bytes
+ * includes room for the trailing update's operands, and caqr_factor accepts
+ * a workspace without it, down to this query's size for a single panel
+ * (n = b), and then updates on the FP64 pipe. */
 int ca_caqr_workspace(int m, int n, int b, const ca_tree_t *tree, size_t *qtree_bytes,
                       size_t *work_bytes);
 
@@ -212,7 +215,8 @@ int calu_getrs(int n, int nrhs, const double *LU, int lda, const int *ipiv, doub
  *   1. TSQR: Householder QR of every leaf, then of every merge node's stacked
  *      upper-triangular R factors (the R-elimination tree);
  *   2. the trailing columns get every leaf's Q^T (UPFACT), then every merge
- *      node's Q^T bottom-up (UPELIM).
+ *      node's Q^T bottom-up (UPELIM); with the queried workspace large updates
+ *      run on the tensor cores from exact digits, as in calu_factor.
  * Q is kept in the compact Y T Y^T form (Sec. 3.1), stored in a tree
  * structure:
  *   - leaf j of panel k: Householder vectors strictly below the leaf-local

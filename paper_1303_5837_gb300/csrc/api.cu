@@ -235,7 +235,7 @@ int calu_run(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, int
 // update of the trailing columns in FP64 (tcws == nullptr) or on the tensor
 // cores.  With look-ahead the per-node arrays alternate between two copies.
 int caqr_run(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, double *qtree, void *work, int nl,
-             void *tcws, int slices, int exact, int *dev_info, cudaStream_t stream) {
+             void *tcws, int slices, int exact, int *dev_info, cudaStream_t stream, void *f64ws = nullptr) {
   if (cudaMemsetAsync(dev_info, 0, 2 * sizeof(int), stream) != cudaSuccess) return CA_ERR_LAUNCH;
   if (n == 0) return CA_OK;
   QrPanelWs wsv[2];
@@ -269,6 +269,9 @@ int caqr_run(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, dou
       if (tcws)
         return tree_apply_qt_tc(mk, bk, b, P, lda, L, plan, Tp, C, lda, ncols, ws, tcws, slices, exact,
                                 dev_info + 1, stream);
+      if (f64ws && tree_tc_pays(mk, bk, ncols, L, plan))
+        return tree_apply_qt_tc(mk, bk, b, P, lda, L, plan, Tp, C, lda, ncols, ws, f64ws, kTcF64Slices, 1,
+                                dev_info + 1, stream, 1);
       return tree_apply_qt(mk, bk, b, P, lda, L, plan, Tp, C, lda, ncols, ws, stream);
     };
     if (nt > 0) {
@@ -295,6 +298,14 @@ cudaError_t getrs_run(int n, int nrhs, const double *LU, int lda, const int *ipi
   if (e != cudaSuccess) return e;
   if ((e = trsm_left(true, true, n, nrhs, LU, lda, B, ldb, sw, status, bit, skip, stream)) != cudaSuccess) return e;
   return trsm_left(false, false, n, nrhs, LU, lda, B, ldb, sw, status, bit, skip, stream);
+}
+
+// Workspace of CAQR's FP64 tree updates on the tensor cores (0 where none of
+// them would run there).
+size_t qr_f64_ws_bytes(int m, int n, int b, const ca_tree_t *tree, int nl) {
+  Plan plan;
+  if (b >= n || !build_plan(nl, *tree, plan) || !tree_tc_pays(m, b, n - b, tree->leaf_rows, plan)) return 0;
+  return tree_tc_ws_bytes(m, b, n - b, tree->leaf_rows, nl, kTcF64Slices);
 }
 
 size_t caqr_mixed_ws(int m, int n, int b, const ca_tree_t *tree, int nl, int slices) {
@@ -353,7 +364,7 @@ int ca_caqr_workspace(int m, int n, int b, const ca_tree_t *tree, size_t *qtree_
   if (rc == -5 || rc == -6) rc = (rc == -5) ? -3 : -4;
   if (rc != CA_OK) return rc;
   *qtree_bytes = q;
-  *work_bytes = 2 * align256(qr_panel_ws_bytes(nl));  // two copies for look-ahead
+  *work_bytes = 2 * align256(qr_panel_ws_bytes(nl)) + qr_f64_ws_bytes(m, n, b, tree, nl);  // two copies for look-ahead
   return CA_OK;
 }
 
@@ -437,7 +448,11 @@ int caqr_factor(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, 
   if (!dev_info) return -11;
   if (n > 0 && (!qtree || qtree_bytes < qneed)) return CA_ERR_WORKSPACE;
   if (n > 0 && (!work || lwork < 2 * align256(qr_panel_ws_bytes(nl)))) return CA_ERR_WORKSPACE;
-  return caqr_run(m, n, A, lda, b, tree, qtree, work, nl, nullptr, 0, 0, dev_info, stream);
+  // as calu_factor: the tree updates run on the tensor cores when the
+  // workspace has room for them
+  const size_t base = 2 * align256(qr_panel_ws_bytes(nl)), more = qr_f64_ws_bytes(m, n, b, tree, nl);
+  void *f64ws = (more > 0 && lwork >= base + more) ? (char *)work + base : nullptr;
+  return caqr_run(m, n, A, lda, b, tree, qtree, work, nl, nullptr, 0, 0, dev_info, stream, f64ws);
 }
 
 int tsqr(int m, int n, double *A, int lda, const ca_tree_t *tree, double *qtree,

@@ -337,7 +337,10 @@ cudaError_t gemm_minus_f64_tc(int m, int n, int k, const double *A, int lda, con
 size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, int S);
 cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, int leaf_rows, const Plan &plan,
                              const double *Tp, double *C, int ldc, int ncols, const QrPanelWs &ws, void *tcws,
-                             int S, int exact, int *status, cudaStream_t st);
+                             int S, int exact, int *status, cudaStream_t st, int full = 0);
+// whether the FP64 update (7 exact digits, full = 1) is faster there than on
+// the FP64 pipe
+bool tree_tc_pays(int mk, int bk, int ncols, int leaf_rows, const Plan &plan);
 
 // triangular solves (solve.cu).  The dependency-ordered solve keeps its
 // ready flags in caller memory (SolveWs, solve_ws_bytes(n) bytes): word 0

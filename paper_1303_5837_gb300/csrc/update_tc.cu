@@ -71,7 +71,7 @@ __global__ void leaf_items_kernel(int nleaves, int L, int mk, int bk, int *top, 
 }
 
 size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, int S) {
-  const int ch = kChunkLeaves;
+  const int ch = nleaves < kChunkLeaves ? nleaves : kChunkLeaves;
   const size_t w = (size_t)ch * bk * ncols * 8;
   size_t g = tc_gemm_ws_bytes_batched(bk, ncols, kHalfK, S, ch);           // W = Y^T C (per half)
   g = g > tc_gemm_ws_bytes_batched(leaf_rows, ncols, bk, S, ch) ? g
@@ -81,12 +81,27 @@ size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, i
   return 2 * align256(w) + align256(g) + items + 256;
 }
 
+// The FP64 tree update from 7 digits: like the Schur update (gemm_tc.cu) its
+// products are exact and its error below that of FP64 multiply-adds.  It is a
+// chain of many small launches (three per contraction of up to 128 rows), so
+// it pays where the FP64 kernels would take longer than about 5 us per launch
+// at the 0.5 TFLOP/s they reach on the shapes near the line (1.07 wide, 0.2
+// narrow).  CAQR of 6144 x 6144 (1024-row leaves): 433 -> 227 ms; 2000 x 2000,
+// b = 64, 128-row leaves: 70.7 -> 64.5 ms, with the line at a fourth of the
+// columns the same, at four times as many 68.3.
+bool tree_tc_pays(int mk, int bk, int ncols, int leaf_rows, const Plan &plan) {
+  int launches = ((leaf_rows + kHalfK - 1) / kHalfK + 2) * 3 + 3;
+  for (int r = 0; r < plan.nrounds; ++r) launches += 3 * (2 * plan.r[r].max_cnt - 1) + 4;
+  const double fp64_us = 4.0 * mk * bk * (double)ncols / 0.5e6;
+  return bk >= 16 && bk <= 128 && fp64_us > 5.0 * launches;
+}
+
 cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, int leaf_rows, const Plan &plan,
                              const double *Tp, double *C, int ldc, int ncols, const QrPanelWs &ws, void *tcws,
-                             int S, int exact, int *status, cudaStream_t st) {
+                             int S, int exact, int *status, cudaStream_t st, int full) {
   if (ncols <= 0) return cudaSuccess;
   const int L = leaf_rows, nl = plan.nleaves;
-  const int ch = kChunkLeaves;
+  const int ch = nl < kChunkLeaves ? nl : kChunkLeaves;  // a round of merges has fewer nodes
   char *p = (char *)(((uintptr_t)tcws + 255) & ~(uintptr_t)255);
   double *W = (double *)p;
   p += align256((size_t)ch * bk * ncols * 8);
@@ -147,6 +162,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
       g1.sign = -1.0;
       g1.S = S;
       g1.exact = exact;
+      g1.full = full;
       if ((e = gemm_tc(g1, gws, status, st)) != cudaSuccess) return e;
     }
     // W' = T^T W
@@ -173,6 +189,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
     g2.sign = -1.0;
     g2.S = S;
     g2.exact = exact;
+    g2.full = full;
     if ((e = gemm_tc(g2, gws, status, st)) != cudaSuccess) return e;
     // C -= Y W'
     TcGemm g3 = {};
@@ -194,6 +211,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
     g3.sign = 1.0;
     g3.S = S;
     g3.exact = exact;
+    g3.full = full;
     if ((e = gemm_tc(g3, gws, status, st)) != cudaSuccess) return e;
   }
 
@@ -247,6 +265,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
         g1.sign = -1.0;
         g1.S = S;
         g1.exact = exact;
+        g1.full = full;
         if ((e = gemm_tc(g1, gws, status, st)) != cudaSuccess) return e;
       }
       TcGemm g2 = {};
@@ -269,6 +288,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
       g2.sign = -1.0;
       g2.S = S;
       g2.exact = exact;
+      g2.full = full;
       if ((e = gemm_tc(g2, gws, status, st)) != cudaSuccess) return e;
       {
         ProfScope ps(kClsTreeApply, st, 0.0);
@@ -295,6 +315,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
         g3.sign = 1.0;
         g3.S = S;
         g3.exact = exact;
+        g3.full = full;
         if ((e = gemm_tc(g3, gws, status, st)) != cudaSuccess) return e;
       }
     }

@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 from paper_1303_5837_gb300 import inputs
-from tests.parity import check, lu_err
+from tests.parity import check, lu_err, qr_err, qtree_err
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -98,3 +98,43 @@ def test_lu_update_of_odd_values_is_the_fp64_pipes(ca, value):
     assert np.array_equal(np.isinf(got[:192]), np.isinf(want[:192]))
     fin = np.isfinite(want[:192])
     assert np.allclose(got[:192][fin], want[:192][fin], rtol=1e-9, atol=1e-9)
+
+
+def qr_run(ca, A, b, tree, single_panel_workspace):
+    m, n = A.shape
+    F = to_dev(A)
+    work = None
+    if single_panel_workspace:
+        work = torch.empty(ca.ca_caqr_workspace(m, b, b, tree)[1] // 8, dtype=torch.float64, device="cuda")
+        assert work.numel() * 8 < ca.ca_caqr_workspace(m, n, b, tree)[1]
+    before = ca.ca_launch_count(9)
+    qtree, info = ca.caqr_factor(F, b, tree, work=work)
+    torch.cuda.synchronize()
+    assert (ca.ca_launch_count(9) > before) != single_panel_workspace
+    return to_host(F), qtree.cpu().numpy(), info.cpu().tolist()
+
+
+@pytest.mark.parametrize("m,n,b,L,lv", [(2000, 1500, 64, 128, [(0, 0)]), (2501, 1111, 100, 300, [(4, 1), (0, 1)]),
+                                        (3000, 1000, 128, 1024, [(0, 1)])])
+def test_qr_update_matches_the_oracle(ca, m, n, b, L, lv):
+    A = inputs.gaussian(m, n, m + n + b)
+    t_o = oracle.make_tree(L, lv)
+    QR_o, T_o = oracle.caqr(A, b, t_o)
+    for alone in (False, True):
+        got, qtree, info = qr_run(ca, A, b, ca.make_tree(L, lv), alone)
+        assert info == [0, 0]
+        check(qr_err(got, QR_o, b), TOL, (m, n, b, alone))
+        check(qtree_err(qtree, T_o, QR_o, b, t_o, oracle.tree_counts), TOL, (m, n, b, alone))
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan, 1e-310])
+def test_qr_update_of_odd_values_is_the_fp64_pipes(ca, value):
+    A = inputs.gaussian(2000, 1400, 5)
+    A[70, 1300] = value
+    t = ca.make_tree(128)
+    got, _, _ = qr_run(ca, A, 64, t, False)
+    want, _, _ = qr_run(ca, A, 64, t, True)
+    clean = np.arange(1280)  # whole panels before the value's column
+    assert np.all(np.isfinite(got[:, clean]) == np.isfinite(want[:, clean]))
+    assert np.array_equal(np.isfinite(got[:1280, 1300]), np.isfinite(want[:1280, 1300]))
+    assert np.allclose(got[:1280][:, clean], want[:1280][:, clean], rtol=1e-9, atol=1e-9)
