@@ -43,6 +43,7 @@
 
 #include "ca_internal.cuh"
 #include "device_once.cuh"
+#include "fp64_int.cuh"
 #include "lu_node.cuh"
 
 namespace cagb {
@@ -131,30 +132,6 @@ __device__ __forceinline__ void warp_best(unsigned long long &key, int &pos) {
 // out of line, so that it is not computed beside the integer form every time
 __device__ __noinline__ double recip_lib(double v) { return __drcp_rn(v); }
 
-// 1 / v without the FP64 pipe: the hardware's single-precision reciprocal of
-// the leading bits (relative error e below 2^-21) and one third-order
-// Householder step x (1 + e + e^2) in 64-bit fixed point.  y = 2^62 / m comes
-// out at most 16 units off (truncations of 1, 4 and 8, and e^3 below 1), so
-// rounding it to 53 bits gives the correctly rounded reciprocal unless its
-// last ten bits lie within 24 of the tie.  Those values (1 in 20), and values
-// near the ends of the range, zeros, infinities and NaN, return 0: the thread
-// that publishes takes the library's reciprocal then.
-__device__ __forceinline__ double recip(double v) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
-  const int E = (int)((bits >> 52) & 0x7ff);
-  const unsigned long long M = bits & ((1ull << 52) - 1);
-  float x;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(__uint_as_float(0x3f800000u | (unsigned)(M >> 29))));
-  const unsigned long long m = (M | (1ull << 52)) << 11;                        // m / 2^64 = |v| / 2^(E - 1022)
-  const unsigned long long x0 = (unsigned long long)(unsigned)(x * 2147483648.0f) << 32;  // 2^62 / that, about
-  const long long e = (long long)((1ull << 62) - __umul64hi(m, x0));             // 2^62 (1 - m x0)
-  const long long f = e + (__mul64hi(e, e) << 2);
-  const unsigned long long y = x0 + (unsigned long long)(__mul64hi(f, (long long)(x0 >> 1)) << 3);
-  const bool sure = (unsigned)(E - 64) < 0x7ffu - 128u && (unsigned)((int)(y & 1023) - 512 + 24) > 48u;
-  const unsigned long long mant = (y + 512) >> 10;                               // in [2^52, 2^53]
-  return !sure ? 0.0 : __longlong_as_double((long long)(((bits >> 63) << 63) | (((unsigned long long)(2044 - E) << 52) + mant)));
-}
-
 template <int TPR, int CPT, bool CL>
 struct Node {
   cg::cluster_group cl;
@@ -196,7 +173,7 @@ struct Node {
   }
 
   // Publishes the CTA's best row of column j: on the warp that holds it
-  // (mine; `lead` holds its leading value v, r = recip(v)), or, without a
+  // (mine; `lead` holds its leading value v, r its reciprocal or 0), or, without a
   // candidate in this CTA, an empty key from warp 0.
   __device__ __forceinline__ void publish(int j, int nb, bool mine, bool lead, double v, double r,
                                           unsigned long long key, int p) {
@@ -291,7 +268,7 @@ struct Node {
       {
         const bool mine = s.key != 0ull && pos == s.p;
         if (__any_sync(0xffffffffu, mine) || (CL && s.key == 0ull && warp == 0)) {
-          if (!s.early) s.r = recip(s.v);
+          if (!s.early) s.r = recip_exact_or_zero(s.v);
           publish(j, nb, mine, mine && sub == h, s.v, s.r, s.key, s.p);
         }
       }
@@ -319,7 +296,7 @@ struct Node {
         post_key(j + 1, cand ? absbits(s.v) : 0ull, cand ? pos : INT_MAX);
       }
       s.aj = TPR > 1 ? __shfl_sync(0xffffffffu, s.v, sn, TPR) : s.v;
-      if (s.early) s.r = recip(s.v);
+      if (s.early) s.r = recip_exact_or_zero(s.v);
       if (act) {
 #pragma unroll
         for (int k = Q + 2; k < 4; ++k) a[k] = fma(-l, u[k], a[k]);
@@ -350,7 +327,7 @@ struct Node {
     s.j = 0;
     s.nb = blocks(0);
     s.v = a[0];
-    s.r = recip(s.v);
+    s.r = recip_exact_or_zero(s.v);
     s.aj = TPR > 1 ? __shfl_sync(0xffffffffu, s.v, 0, TPR) : s.v;
     // few warps: every warp has its own candidate's reciprocal ready when the
     // best is known; many: one warp forms it then, and the others keep the

@@ -935,8 +935,8 @@ cudaError_t tsqr_panel(int mk, int bk, int b, double *P, int lda, int leaf_rows,
   // G = 0: the register-resident node kernel; -1: its cluster form; else
   // the shared-memory node kernel on a cluster of G CTAs
   auto pick = [&](int rows, int nodes) {
+    if (tsqr_creg_fits(rows, bk, nodes)) return -1;
     if (tsqr_reg_fits(rows, bk)) return 0;
-    if (tsqr_creg_cluster(rows, bk) >= 2) return -1;
     const int g = pick_qr_cluster(rows, bk, nodes, &rloc, &ld);
     return g > 0 ? g : -2;
   };
