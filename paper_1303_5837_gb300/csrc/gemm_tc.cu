@@ -31,6 +31,7 @@
 #include <cuda_bf16.h>
 
 #include <climits>
+#include <type_traits>
 
 #include "ca_internal.cuh"
 #include "device_once.cuh"
@@ -214,6 +215,40 @@ __device__ __forceinline__ double scaled_rn(long long v, int e2) {
   const int E = (int)((bits >> 52) & 0x7ff) + e2;
   if (v != 0 && E > 0 && E < 2047) return __longlong_as_double(bits + ((long long)e2 << 52));
   return i64_scaled_to_double(v, e2);
+}
+
+// (hi 2^16 + lo) 2^e2 as a double, rounded once to nearest even, |hi| < 2^60
+// and |lo| < 2^40: the sum is brought to 64 normalized bits with a sticky last
+// one and rounded in integers, so the only FP64 instruction left is the
+// subtraction from C (7 digits: 119.6 -> 114.9 ms of updates at n = 10240;
+// with at most 5 digits one conversion of hi is cheaper).
+__device__ __forceinline__ double scaled_sum_rn(long long hi, long long lo, int e2) {
+  hi += lo >> 16;                                  // floor: lo's low 16 bits stay non-negative
+  unsigned long long w = (unsigned long long)(lo & 0xffff) << 48;  // bits below hi
+  unsigned long long h = (unsigned long long)hi;
+  const unsigned long long sign = h & (1ull << 63);
+  if (sign) {                                      // two's complement of the pair
+    w = 0ull - w;
+    h = ~h + (w == 0ull);
+  }
+  if (h == 0ull) {                                 // fewer than 17 bits (or none)
+    const double v = i64_scaled_to_double((long long)(w >> 48), e2);
+    return __longlong_as_double((long long)((unsigned long long)__double_as_longlong(v) | (v != 0.0 ? sign : 0ull)));
+  }
+  const int lz = __clzll((long long)h);            // >= 3
+  unsigned long long n = (h << lz) | (w >> (64 - lz));
+  n |= (w << lz) != 0ull;
+  // n in [2^63, 2^64): value n 2^(e2 + 16 - lz), 53 bits kept
+  const int E = 1023 + 63 + 16 - lz + e2;
+  if ((unsigned)(E - 1) >= 2045u) {                // outside the normal range: the slow path
+    const double v = i64_scaled_to_double((long long)(n >> 2) | (long long)((n & 3) != 0), e2 + 18 - lz);
+    return __longlong_as_double((long long)((unsigned long long)__double_as_longlong(v) | sign));
+  }
+  unsigned long long m = n >> 11;
+  const unsigned rem = (unsigned)n & 0x7ffu;
+  m += (rem > 0x400u || (rem == 0x400u && (m & 1ull))) ? 1ull : 0ull;
+  // a carry out of the 53 bits lands in the exponent
+  return __longlong_as_double((long long)(sign | (((unsigned long long)(E - 1) << 52) + m)));
 }
 
 // Digits of x for the split: F = round(|x| 2^(8S - e)) (|x| < 2^e), as a
@@ -417,8 +452,7 @@ __global__ void __launch_bounds__(256, 2)
     // exact mode: the digit diagonals D = 0 .. S-1 (weights 2^(-8 D)) are
     // integers below 2^24; combine them in integer arithmetic,
     //   T_hi = sum_{D <= 4} acc_D 2^(8 (4 - D)),  T_lo = sum_{D > 4} acc_D 2^(8 (6 - D)),
-    // and turn each into a double by one correctly rounded conversion and an
-    // exponent add (FP64 pipe: the conversion and the subtraction from C).
+    // and round their sum to a double once.
     const int dmax = a.exact ? a.S - 1 : 0;
     constexpr int kEp = 8;  // columns per epilogue step
     for (int c0 = half * kEp; c0 < a.bn; c0 += 2 * kEp) {
@@ -469,8 +503,10 @@ __global__ void __launch_bounds__(256, 2)
         } else if (a.exact) {
           // value = T_hi 2^(8 (4 - dmax)) ... written relative to diagonal dmax:
           // sum_D acc_D 2^(-8 D) = T_hi 2^(-32) + T_lo 2^(-48)
-          c -= scaled_rn(a.sign > 0 ? thi[j] : -thi[j], sc - 32);
-          if (dmax > 4) c -= scaled_rn(a.sign > 0 ? tlo[j] : -tlo[j], sc - 48);
+          if (dmax > 4)
+            c -= scaled_sum_rn(a.sign > 0 ? thi[j] : -thi[j], a.sign > 0 ? tlo[j] : -tlo[j], sc - 48);
+          else
+            c -= scaled_rn(a.sign > 0 ? thi[j] : -thi[j], sc - 32);
         } else {
           c = fma((double)(-a.sign * vf[j]), pow2i(sc), c);
         }
@@ -497,9 +533,10 @@ __global__ void __launch_bounds__(256, 2)
 // 2 upper (r <= q stored); (r, q) = (v + roff, k) or, transposed, (k + roff, v).
 // Output: out[((b * S + s) * vpad + v) * kpad + k], exponent ex[b * vpad + v].
 // --------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int S, int vpad, int kpad, int exact,
+template <bool FULL, int S>
+__global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int vpad, int kpad, int exact,
                                                     __nv_bfloat16 *__restrict__ out, int *__restrict__ ex,
-                                                    const int *skip, int full, const int *kexp, int ksign) {
+                                                    const int *skip, const int *kexp, int ksign) {
   if (skip && *skip) return;
   const int lane = threadIdx.x & 31;
   const int v = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -524,7 +561,7 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
     const unsigned long long bits = absbits(val);
     mx = bits > mx ? bits : mx;
     sh[t] = 0;
-    if (full) {
+    if constexpr (FULL) {
       if (kexp && k < K) sh[t] = ksign * kexp[k];
       if (bits != 0) me = max(me, (int)(bits >> 52) + sh[t]);
       odd |= (bits >> 52) == 0x7ffull;
@@ -541,7 +578,7 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
     const int E = (int)(mx >> 52);
     e = (E == 0) ? -1021 : E - 1022;
   }
-  if (full) {
+  if constexpr (FULL) {
     me = __reduce_max_sync(0xffffffffu, me);
     odd = __reduce_or_sync(0xffffffffu, odd);
     if (mx != 0) {
@@ -559,26 +596,21 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
     const int k = lane + 32 * t;
     if (k >= kpad) continue;
     // F = round(x 2^(8S - e)) = sum_s d_s 256^(S-1-s), balanced digits
-    // d_s in [-128, 127] for s >= 1 and |d_0| <= 256, all integer arithmetic
-    long long F = fixed_point_digits(x[t], e - sh[t], S);
-    int dg[8];
+    // d_s in [-128, 127] for s >= 1 and |d_0| <= 256: with 128 added at every
+    // lower digit's place, the bytes of F are d_s + 128 and what is above them
+    // is d_0.  A byte becomes a float by putting it into the mantissa of 2^23
+    // (no conversion instruction).
+    constexpr unsigned long long bias = 0x0080808080808080ull & ((1ull << (8 * (S - 1))) - 1);
+    const unsigned long long F = (unsigned long long)fixed_point_digits(x[t], FULL ? e - sh[t] : e, S) + bias;
 #pragma unroll
-    for (int s = 7; s >= 1; --s) {
-      if (s >= S) continue;
-      int d = (int)(F & 255);
-      if (d >= 128) d -= 256;
-      dg[s] = d;
-      F = (F - d) >> 8;
-    }
-    dg[0] = (int)F;
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      if (s >= S) break;
+    for (int s = 0; s < S; ++s) {
+      const int sft = 8 * (S - 1 - s);
+      const float d = s == 0 ? (float)(int)((long long)F >> sft)
+                             : __uint_as_float(0x4b000000u | (unsigned)((F >> sft) & 255u)) - (8388608.0f + 128.0f);
       // stored value: d_s (exact mode) or d_s 2^(-8 s) (fused mode), exact in bf16
       // 2^(-8 s) as a float from its exponent field (s <= 7: a normal number)
       const float w = exact ? 1.0f : __int_as_float((127 - 8 * s) << 23);
-      const float val = (float)dg[s] * w;
-      out[(((long long)b * S + s) * vpad + v) * kpad + k] = __float2bfloat16_rn(val);
+      out[(((long long)b * S + s) * vpad + v) * kpad + k] = __float2bfloat16_rn(d * w);
     }
   }
 }
@@ -718,16 +750,29 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
   __nv_bfloat16 *sb = (__nv_bfloat16 *)p;
   p += align256(nb * S * np * kp * 2);
   int *eb = (int *)p;
-  if (!g.reuse_a) {
+  auto split = [&](const TcOperand &o, int vpad, __nv_bfloat16 *out, int *ex, int ksign) {
     ProfScope ps(kClsSplit, st, 0.0);
-    split_kernel<<<dim3((mp + 7) / 8, g.nbatch), 256, 0, st>>>(g.A, g.nbatch, S, mp, kp, exact, sa, ea,
-                                                                g.skip, g.full, g.kexp, -1);
-  }
-  {
-    ProfScope ps(kClsSplit, st, 0.0);
-    split_kernel<<<dim3((np + 7) / 8, g.nbatch), 256, 0, st>>>(g.B, g.nbatch, S, np, kp, exact, sb, eb,
-                                                                g.skip, g.full, g.kexp, 1);
-  }
+    const dim3 grid((vpad + 7) / 8, g.nbatch);
+    auto run = [&](auto slices) {
+      constexpr int kS = decltype(slices)::value;
+      if (g.full)
+        split_kernel<true, kS><<<grid, 256, 0, st>>>(o, g.nbatch, vpad, kp, exact, out, ex, g.skip, g.kexp, ksign);
+      else
+        split_kernel<false, kS><<<grid, 256, 0, st>>>(o, g.nbatch, vpad, kp, exact, out, ex, g.skip, nullptr, 0);
+    };
+    switch (S) {
+      case 1: run(std::integral_constant<int, 1>()); break;
+      case 2: run(std::integral_constant<int, 2>()); break;
+      case 3: run(std::integral_constant<int, 3>()); break;
+      case 4: run(std::integral_constant<int, 4>()); break;
+      case 5: run(std::integral_constant<int, 5>()); break;
+      case 6: run(std::integral_constant<int, 6>()); break;
+      case 7: run(std::integral_constant<int, 7>()); break;
+      default: run(std::integral_constant<int, 8>()); break;
+    }
+  };
+  if (!g.reuse_a) split(g.A, mp, sa, ea, -1);
+  split(g.B, np, sb, eb, 1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   CUtensorMap ma, mb;
