@@ -349,7 +349,7 @@ bool tree_tc_pays(int mk, int bk, int ncols, int leaf_rows, const Plan &plan);
 // skip: as for gemm_minus_f64.
 struct SolveWs {
   int *status;
-  int *flags;
+  unsigned char *flags;
 };
 size_t solve_ws_bytes(int n);
 void solve_ws_carve(void *w, int n, SolveWs &s);

@@ -108,12 +108,16 @@ __global__ void __launch_bounds__(256) trsm_diag_kernel(int nb, int nrhs, const 
 // ---------------------------------------------------------------------------
 // Few right-hand sides: one cooperative launch, one CTA per diagonal block,
 // ordered by per-block ready flags instead of grid-wide barriers.
-//   Phase 0: CTA c inverts diagonal block c of T in its shared memory
-//            (LAPACK trti2 order, unit lower or non-unit upper).
+//   Phase 0: CTA c loads diagonal block c of T and inverts its four 32 x 32
+//            diagonal sub-blocks, one warp each (one per SM sub-partition; a
+//            lane per column, the column in registers).
 //   Then CTA c takes the blocks it depends on in order (the ones before it
 //   for L, after it for U): it waits until block j's solution is published
 //   (flag j), subtracts T(c, j) x_j from its right-hand sides, and after the
-//   last one computes x_c = T_cc^-1 b_c, writes it to B and publishes flag c.
+//   last one solves T_cc x_c = b_c by sub-blocks, writes it to B and publishes
+//   flag c.  (Inverting the whole 128 x 128 block took 0.85 ms of dependent
+//   multiply-adds per triangle, whatever its order; the sub-blocks 16 us, and
+//   the substitution over them as long as the product with the inverse did.)
 //   The chain of dependent steps is one GEMV of a 128 x 128 block and one
 //   small triangular multiply per block; the earlier GEMVs of a CTA overlap
 //   with the chain.  The cooperative launch makes every CTA resident, as the
@@ -125,7 +129,6 @@ __global__ void __launch_bounds__(256) trsm_diag_kernel(int nb, int nrhs, const 
 // Needs one CTA per diagonal block: n <= SMs * kTb.
 // ---------------------------------------------------------------------------
 constexpr int kCoopMaxRhs = 16;
-constexpr int kLdI = kTb + 1;
 constexpr int kMaxFlagBlocks = 1024;            // flag words of a solve workspace (covers any SM count here)
 constexpr long long kSolveWaitLimit = 4000000000ll;
 
@@ -134,18 +137,20 @@ constexpr long long kSolveWaitLimit = 4000000000ll;
 static std::atomic<long long> g_wait_limit{kSolveWaitLimit};
 static std::atomic<int> g_withhold{-1};
 
-__device__ __forceinline__ int ld_acquire_gpu(const int *p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+// ready flags: one byte per diagonal block (the workspace has room for 4 bytes
+// per 128 rows, whichever block size a solve uses)
+__device__ __forceinline__ int ld_acquire_gpu(const unsigned char *p) {
+  unsigned short v;
+  asm volatile("ld.acquire.gpu.global.u8 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
   return v;
 }
 
-__device__ __forceinline__ void st_release_gpu(int *p, int v) {
-  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void st_release_gpu(unsigned char *p) {
+  asm volatile("st.release.gpu.global.u8 [%0], %1;" ::"l"(p), "h"((unsigned short)1) : "memory");
 }
 
 struct FlagArgs {
-  int *flags;            // nblk ready flags, zero at launch
+  unsigned char *flags;  // nblk ready flags, zero at launch
   int *status;           // gets status_bit when a wait gives up
   int status_bit;
   const int *skip;       // refinement: nonzero = the loop has stopped, do nothing
@@ -153,81 +158,77 @@ struct FlagArgs {
   int withhold_blk;      // test hook (-1: off)
 };
 
+constexpr int kTs = 32;  // sub-block of a diagonal block
+
+// Column `lane` of the inverse of the kTs x kTs triangle at Ti (ld kLdI,
+// zeros outside it, a nonzero diagonal), by substitution on a unit vector.
+template <bool LOWER, int kLdI>
+__device__ __forceinline__ void invert_sub(double *Ti, bool unit, int lane) {
+  double x[kTs];
+#pragma unroll
+  for (int i = 0; i < kTs; ++i) x[i] = (i == lane) ? 1.0 : 0.0;
+  const double rd = unit ? 1.0 : 1.0 / Ti[lane + lane * kLdI];
+#pragma unroll
+  for (int s = 0; s < kTs; ++s) {
+    const int k = LOWER ? s : kTs - 1 - s;
+    const double r = __shfl_sync(0xffffffffu, rd, k);
+    if (!unit) x[k] *= r;
+#pragma unroll
+    for (int i = 0; i < kTs; ++i)
+      if (LOWER ? i > k : i < k) x[i] = fma(-Ti[i + k * kLdI], x[k], x[i]);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < kTs; ++i) Ti[i + lane * kLdI] = x[i];
+}
+
+template <bool LOWER, int kTb>
 __global__ void __launch_bounds__(256, 1) trsv_flag_kernel(int n, int nrhs, const double *T, int ldt, double *B,
-                                                           int ldb, int lower, int unit, FlagArgs fa) {
+                                                           int ldb, int unit, FlagArgs fa) {
   extern __shared__ __align__(16) double csm[];
-  double *Ti = csm;                          // the inverted diagonal block, ld kLdI
-  double *tmp = Ti + kTb * kLdI;             // kTb column buffer
-  double *sb = tmp + kTb;                    // kTb x nrhs: my right-hand sides being reduced
+  constexpr bool lower = LOWER;
+  constexpr int kLdI = kTb + 1;
+  constexpr int kParts = 256 / kTb, kKp = kTb / kParts;  // threads per row of a block product, columns each
+  double *Ti = csm;                          // the diagonal block, its sub-blocks inverted, ld kLdI
+  double *sb = Ti + kTb * kLdI;                   // kTb x nrhs: my right-hand sides being reduced
   double *xj = sb + kTb * kCoopMaxRhs;       // kTb x nrhs: a published solution block
-  double *part = xj + kTb * kCoopMaxRhs;     // 2 x kTb x nrhs: half-row partial sums
+  double *part = xj + kTb * kCoopMaxRhs;     // kParts x kTb x nrhs: partial sums of the rows
   __shared__ int abort_flag;
   if (fa.skip && *fa.skip) return;
-  int *flags = fa.flags;
+  unsigned char *flags = fa.flags;
   const int tid = threadIdx.x;
   const int nblk = (n + kTb - 1) / kTb;
   const int blk = blockIdx.x;
   if (blk >= nblk) return;
   const int r0 = blk * kTb, nb = min(kTb, n - r0);
 
-  // ---- phase 0: invert my diagonal block ----------------------------------
-  for (int idx = tid; idx < nb * nb; idx += blockDim.x) {
-    const int i = idx % nb, k = idx / nb;
-    const bool keep = lower ? (i >= k) : (i <= k);
-    Ti[i + k * kLdI] = keep ? T[(r0 + i) + (size_t)(r0 + k) * ldt] : 0.0;
+  // ---- phase 0: my diagonal block (the identity beyond its rows) and the
+  //      inverses of its diagonal sub-blocks ---------------------------------
+  for (int idx = tid; idx < kTb * kTb; idx += blockDim.x) {
+    const int i = idx % kTb, k = idx / kTb;
+    const bool keep = i < nb && k < nb && (lower ? (i >= k) : (i <= k));
+    Ti[i + k * kLdI] = keep ? T[(r0 + i) + (size_t)(r0 + k) * ldt] : (i == k ? 1.0 : 0.0);
   }
-  for (int idx = tid; idx < nb * nrhs; idx += blockDim.x) {
-    const int k = idx % nb, c = idx / nb;
-    sb[k + c * kTb] = B[(r0 + k) + (size_t)c * ldb];
+  for (int idx = tid; idx < kTb * nrhs; idx += blockDim.x) {
+    const int k = idx % kTb, c = idx / kTb;
+    sb[k + c * kTb] = k < nb ? B[(r0 + k) + (size_t)c * ldb] : 0.0;
   }
   __syncthreads();
-  if (lower) {
-    // lower: columns right to left; X(j, j) = 1 / T(j, j) (1 when unit),
-    // X(j+1:, j) = -X(j+1:, j+1:) T(j+1:, j) X(j, j)
-    for (int i = tid; i < nb; i += blockDim.x) xj[i] = unit ? 1.0 : 1.0 / Ti[i + i * kLdI];
-    __syncthreads();
-    for (int j = nb - 1; j >= 0; --j) {
-      const double djj = xj[j];
-      for (int i = j + 1 + tid; i < nb; i += blockDim.x) {
-        double acc = 0.0;
-        for (int k = j + 1; k <= i; ++k) acc = fma(Ti[i + k * kLdI], Ti[k + j * kLdI], acc);
-        tmp[i] = -acc * djj;
-      }
-      __syncthreads();
-      for (int i = j + 1 + tid; i < nb; i += blockDim.x) Ti[i + j * kLdI] = tmp[i];
-      if (tid == 0) Ti[j + j * kLdI] = djj;
-      __syncthreads();
-    }
-  } else {
-    // non-unit upper: columns left to right; X(j, j) = 1 / T(j, j),
-    // X(0:j, j) = -X(j, j) X(0:j, 0:j) T(0:j, j)
-    for (int i = tid; i < nb; i += blockDim.x) xj[i] = 1.0 / Ti[i + i * kLdI];  // all pivots at once
-    __syncthreads();
-    for (int j = 0; j < nb; ++j) {
-      const double djj = xj[j];
-      for (int i = tid; i < j; i += blockDim.x) {
-        double acc = 0.0;
-        for (int k = i; k < j; ++k) acc = fma(Ti[i + k * kLdI], Ti[k + j * kLdI], acc);
-        tmp[i] = -djj * acc;
-      }
-      __syncthreads();
-      for (int i = tid; i < j; i += blockDim.x) Ti[i + j * kLdI] = tmp[i];
-      if (tid == 0) Ti[j + j * kLdI] = djj;
-      __syncthreads();
-    }
-  }
+  if ((tid >> 5) * kTs < nb && (tid >> 5) < kTb / kTs)
+    invert_sub<LOWER, kLdI>(Ti + (tid >> 5) * kTs * (kLdI + 1), unit != 0, tid & 31);
+  __syncthreads();
 
   // ---- the blocks this one depends on, in order ----------------------------
   const int ndep = lower ? blk : nblk - 1 - blk;
-  const int r = tid & (kTb - 1), half = tid >> 7;  // row of my block, half of the columns
+  const int r = tid & (kTb - 1), half = tid / kTb;  // row of my block, share of the columns
   for (int t = 0; t < ndep; ++t) {
     const int j = lower ? t : nblk - 1 - t;
     const int c0 = j * kTb, nbj = min(kTb, n - c0);
     // prefetch this thread's half row of T(blk, j) while waiting
-    double trow[kTb / 2];
-    const int k0 = half * (kTb / 2);
+    double trow[kKp];
+    const int k0 = half * kKp;
 #pragma unroll
-    for (int k = 0; k < kTb / 2; ++k)
+    for (int k = 0; k < kKp; ++k)
       trow[k] = (r < nb && k0 + k < nbj) ? T[(r0 + r) + (size_t)(c0 + k0 + k) * ldt] : 0.0;
     if (tid == 0) {
       const long long tstart = clock64();
@@ -251,14 +252,14 @@ __global__ void __launch_bounds__(256, 1) trsv_flag_kernel(int n, int nrhs, cons
     if (nrhs == 1) {  // one right-hand side: four independent partial sums
       double a4[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-      for (int k = 0; k < kTb / 2; ++k) a4[k & 3] = fma(trow[k], xj[k0 + k], a4[k & 3]);
+      for (int k = 0; k < kKp; ++k) a4[k & 3] = fma(trow[k], xj[k0 + k], a4[k & 3]);
       part[half * kTb * kCoopMaxRhs + r] = (a4[0] + a4[1]) + (a4[2] + a4[3]);
     } else {
       double acc[kCoopMaxRhs];
 #pragma unroll
       for (int c = 0; c < kCoopMaxRhs; ++c) acc[c] = 0.0;
 #pragma unroll
-      for (int k = 0; k < kTb / 2; ++k) {
+      for (int k = 0; k < kKp; ++k) {
         const double tv = trow[k];
 #pragma unroll
         for (int c = 0; c < kCoopMaxRhs; ++c)
@@ -271,21 +272,60 @@ __global__ void __launch_bounds__(256, 1) trsv_flag_kernel(int n, int nrhs, cons
     __syncthreads();
     for (int idx = tid; idx < nb * nrhs; idx += blockDim.x) {
       const int i = idx % nb, c = idx / nb;
-      sb[i + c * kTb] -= part[i + c * kTb] + part[kTb * kCoopMaxRhs + i + c * kTb];
+      double v = part[i + c * kTb];
+#pragma unroll
+      for (int h = 1; h < kParts; ++h) v += part[h * kTb * kCoopMaxRhs + i + c * kTb];
+      sb[i + c * kTb] -= v;
     }
     __syncthreads();
   }
 
-  // ---- x = T_blk^-1 b_blk, published ---------------------------------------
-  for (int idx = tid; idx < nb * nrhs; idx += blockDim.x) {
-    const int i = idx % nb, c = idx / nb;
-    double acc = 0.0;
-    for (int k = 0; k < nb; ++k) acc = fma(Ti[i + k * kLdI], sb[k + c * kTb], acc);
-    B[(r0 + i) + (size_t)c * ldb] = acc;
+  // ---- T_blk x = b_blk by sub-blocks, published ----------------------------
+  // x_s = (inverse of sub-block s) b_s: 8 threads per row; then the rows still
+  // to come lose their part: kParts threads per row
+  const int nsub = (nb + kTs - 1) / kTs;
+  for (int t = 0; t < nsub; ++t) {
+    const int s0 = (lower ? t : nsub - 1 - t) * kTs;
+    {
+      const int i = tid >> 3, k0 = 4 * (tid & 7);
+      for (int c = 0; c < nrhs; ++c) {
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc = fma(Ti[s0 + i + (s0 + k0 + k) * kLdI], sb[s0 + k0 + k + c * kTb], acc);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((tid & 7) == 0) {
+          xj[i + c * kTs] = acc;
+          if (s0 + i < nb) B[(r0 + s0 + i) + (size_t)c * ldb] = acc;
+        }
+      }
+    }
+    __syncthreads();
+    if (t + 1 < nsub) {
+      constexpr int kKs = kTs / kParts;
+      const int i = tid / kParts, k0 = kKs * (tid % kParts);
+      // whole warps (8 or 16 rows) are on one side of s0: no divergence at the shuffle
+      if (i < nsub * kTs && (lower ? i >= s0 + kTs : i < s0)) {
+        const unsigned m = __activemask();
+        for (int c = 0; c < nrhs; ++c) {
+          double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+          for (int k = 0; k < kKs; k += 2) {
+            a0 = fma(Ti[i + (s0 + k0 + k) * kLdI], xj[k0 + k + c * kTs], a0);
+            a1 = fma(Ti[i + (s0 + k0 + k + 1) * kLdI], xj[k0 + k + 1 + c * kTs], a1);
+          }
+          a0 += a1;
+#pragma unroll
+          for (int o = kParts / 2; o > 0; o >>= 1) a0 += __shfl_xor_sync(m, a0, o);
+          if (tid % kParts == 0) sb[i + c * kTb] -= a0;
+        }
+      }
+      __syncthreads();
+    }
   }
   __threadfence();
   __syncthreads();
-  if (tid == 0 && blk != fa.withhold_blk) st_release_gpu(flags + blk, 1);
+  if (tid == 0 && blk != fa.withhold_blk) st_release_gpu(flags + blk);
 }
 
 // Solve workspace (caller memory): word 0 is the timeout record of the
@@ -298,7 +338,7 @@ size_t solve_ws_bytes(int n) {
 void solve_ws_carve(void *w, int n, SolveWs &s) {
   (void)n;
   s.status = (int *)w;
-  s.flags = (int *)w + 32;
+  s.flags = (unsigned char *)((int *)w + 32);
 }
 
 void solve_test_hook(long long wait_cycles, int withhold_blk) {
@@ -313,18 +353,21 @@ static int coop_max_n() {
   return (sms < kMaxFlagBlocks ? sms : kMaxFlagBlocks) * kTb;
 }
 
+template <int TB>
 static cudaError_t trsm_left_flags(bool lower, bool unit, int n, int nrhs, const double *T, int ldt, double *B,
                                    int ldb, const SolveWs &ws, int *status, int status_bit, const int *skip,
                                    cudaStream_t st) {
   static std::atomic<unsigned long long> init{0};
-  const size_t smem = ((size_t)kTb * kLdI + kTb + 4 * (size_t)kTb * kCoopMaxRhs) * 8;
+  const size_t smem = ((size_t)TB * (TB + 1) + (2 + 256 / TB) * (size_t)TB * kCoopMaxRhs) * 8;
   cudaError_t e = once_per_device(init, [smem] {
-    return cudaFuncSetAttribute(trsv_flag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t r = cudaFuncSetAttribute(trsv_flag_kernel<true, TB>, a, (int)smem);
+    if (r != cudaSuccess) return r;
+    return cudaFuncSetAttribute(trsv_flag_kernel<false, TB>, a, (int)smem);
   });
   if (e != cudaSuccess) return e;
-  const int nblk = (n + kTb - 1) / kTb;
-  e = cudaMemsetAsync(ws.flags, 0, (size_t)nblk * sizeof(int), st);
-  if (e != cudaSuccess) return e;
+  const int nblk = (n + TB - 1) / TB;
+  if (nblk > 1 && (e = cudaMemsetAsync(ws.flags, 0, (size_t)nblk, st)) != cudaSuccess) return e;
   FlagArgs fa;
   fa.flags = ws.flags;
   fa.status = status;
@@ -333,17 +376,28 @@ static cudaError_t trsm_left_flags(bool lower, bool unit, int n, int nrhs, const
   fa.wait_limit = g_wait_limit.load();
   fa.withhold_blk = g_withhold.load();
   if (fa.withhold_blk >= 0) fa.withhold_blk = lower ? 0 : nblk - 1;  // the block nothing else precedes
-  int lo = lower ? 1 : 0, un = unit ? 1 : 0;
-  void *args[] = {&n, &nrhs, (void *)&T, &ldt, &B, &ldb, &lo, &un, &fa};
+  int un = unit ? 1 : 0;
+  void *args[] = {&n, &nrhs, (void *)&T, &ldt, &B, &ldb, &un, &fa};
+  void *fn = lower ? (void *)trsv_flag_kernel<true, TB> : (void *)trsv_flag_kernel<false, TB>;
   ProfScope ps(kClsSolve, st, (double)n * n * nrhs);
-  return cudaLaunchCooperativeKernel((void *)trsv_flag_kernel, dim3(nblk), dim3(256), args, smem, st);
+  if (nblk == 1) return cudaLaunchKernel(fn, dim3(1), dim3(256), args, smem, st);  // waits for nobody
+  return cudaLaunchCooperativeKernel(fn, dim3(nblk), dim3(256), args, smem, st);
 }
 
 cudaError_t trsm_left(bool lower, bool unit, int n, int nrhs, const double *T, int ldt, double *B, int ldb,
                       const SolveWs &ws, int *status, int status_bit, const int *skip, cudaStream_t st) {
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
-  if (nrhs <= kCoopMaxRhs && n > kTb && n <= coop_max_n())
-    return trsm_left_flags(lower, unit, n, nrhs, T, ldt, B, ldb, ws, status, status_bit, skip, st);
+  // up to 16 right-hand sides: one launch per triangle
+  // Blocks of 64 rows while there is an SM for each: the chain is one block
+  // product and one block solve per block on a single SM's FP64 pipe, so twice
+  // the blocks of a quarter the work each (order 2048, 4 right-hand sides: 925
+  // us a triangle before, 750 with blocks of 128, 440 with 64).  A single block
+  // of up to 128 rows has no chain.
+  if (nrhs <= kCoopMaxRhs && n <= coop_max_n()) {
+    if (n > kTb && n <= coop_max_n() / 2)
+      return trsm_left_flags<64>(lower, unit, n, nrhs, T, ldt, B, ldb, ws, status, status_bit, skip, st);
+    return trsm_left_flags<kTb>(lower, unit, n, nrhs, T, ldt, B, ldb, ws, status, status_bit, skip, st);
+  }
   const size_t smem = ((size_t)kTb * (kTb + 1) + (size_t)kTb * 33) * 8;
   static std::atomic<unsigned long long> init{0};
   cudaError_t e = once_per_device(init, [smem] {
