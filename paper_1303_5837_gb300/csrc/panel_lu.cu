@@ -421,81 +421,112 @@ __global__ void __launch_bounds__(256) laswp_kernel(int ncols, double *A, int ld
 }
 
 // ---------------------------------------------------------------------------
-// Panel finish: the top bk x bk block <- L11\U11 of the root; the rows below
-// get L21 = A21 U11^-1 (Sec. 3.2, block column of L).  Right-looking
-// substitution on a tile of rows in shared memory.
+// The triangular solves of a panel, one kernel for both (Sec. 3.2): the rows
+// of L21 = A21 U11^-1 (ROWS) and the columns of U12 = L11^-1 A12 (unit lower).
+// Every vector is on its own: element j becomes final (times 1 / u_jj for
+// ROWS), then element k > j loses x_j times the triangle's element (j, k).
+// TPR threads hold one vector, thread `sub` its elements k TPR + sub, k < CPT,
+// in registers; x_j goes round by a shuffle, the triangle's rows come from
+// shared memory, and there is no barrier after the triangle has been loaded.
+// Bound by the FP64 pipe for many vectors, by the chain of K multiplies,
+// shuffles and multiply-adds (250 clocks a step) for few; the kernels before
+// kept the vectors in shared memory with two barriers and two more shared
+// accesses per multiply-add.  The operations on every element are the same.
+// A launch in CALU of 1024 x 1024: L21 83 -> 20 us, U12 35 -> 12 us; of n =
+// 10240: 264 -> 142 and 131 -> 79 us on average.
+// Registers move down by 4 after 4 TPR elements, as in panel_lu_reg.cu.
 // ---------------------------------------------------------------------------
-constexpr int kFinThreads = 256;
+constexpr int kTriThreads = 256;
 
-__global__ void __launch_bounds__(kFinThreads) lu_finish_kernel(int mk, int bk, double *P, int lda,
-                                                                const double *lu11, int ldl,
-                                                                int rt, const int *skip) {
-  extern __shared__ __align__(16) double fsm[];
+template <int TPR, int CPT, bool ROWS>
+struct TriSolve {
+  const double *C;   // the triangle: row j at j (TPR CPT), blocks of 4 registers by sub
+  const double *rd;  // ROWS: 1 / u_jj
+  int K, sub;
+  double a[CPT];
+
+  template <int Q>
+  __device__ __forceinline__ bool group(int &j, int nb, double *out, size_t step, bool live) {
+#pragma unroll 1
+    for (int h = 0; h < TPR; ++h, ++j) {
+      if (j >= K) break;
+      if (ROWS && sub == h) a[Q] *= rd[j];
+      const double x = __shfl_sync(0xffffffffu, a[Q], h, TPR);
+      // the row's part from the current block on
+      const double *c = C + (size_t)j * (TPR * CPT) + 4 * TPR * (j / (4 * TPR)) + 4 * sub;
+      if (sub > h) a[Q] = fma(-x, c[Q], a[Q]);
+#pragma unroll
+      for (int k = Q + 1; k < 4; ++k) a[k] = fma(-x, c[k], a[k]);
+#pragma unroll
+      for (int b = 1; b < CPT / 4; ++b) {
+        if (b >= nb) break;
+        const double2 w0 = *reinterpret_cast<const double2 *>(c + 4 * TPR * b);
+        const double2 w1 = *reinterpret_cast<const double2 *>(c + 4 * TPR * b + 2);
+        a[4 * b] = fma(-x, w0.x, a[4 * b]);
+        a[4 * b + 1] = fma(-x, w0.y, a[4 * b + 1]);
+        a[4 * b + 2] = fma(-x, w1.x, a[4 * b + 2]);
+        a[4 * b + 3] = fma(-x, w1.y, a[4 * b + 3]);
+      }
+    }
+    const int e = (j - 1) / TPR * TPR + sub;  // the elements that are final now
+    if (live && e < K) out[(size_t)e * step] = a[Q];
+    return j < K;
+  }
+};
+
+template <int TPR, int CPT, bool ROWS>
+__global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(int nv, int K, const double *M, int ldm, double *X,
+                                                                int ldx, int vb, double *top, int ldt,
+                                                                const int *skip) {
+  extern __shared__ __align__(16) double tsm[];
   if (skip && *skip) return;
-  // U's upper triangle packed by rows: row j (columns j .. bk-1) at uoff(j)
-  double *U = fsm;
-  double *rd = U + (size_t)bk * (bk + 1) / 2;  // reciprocals of U's diagonal
-  double *T = rd + bk;                         // rt x bk tile (ld rt)
-  auto uoff = [bk](int j) { return j * bk - j * (j - 1) / 2; };
   const int tid = threadIdx.x;
-  if (blockIdx.x == 0) {
-    for (int k = 0; k < bk; ++k)
-      for (int i = tid; i < bk; i += kFinThreads) P[i + (size_t)k * lda] = lu11[i + (size_t)k * ldl];
+  if (ROWS && blockIdx.x == gridDim.x - 1) {  // L11 \ U11 of the root into its place
+    for (int idx = tid; idx < K * K; idx += kTriThreads) {
+      const int i = idx % K, k = idx / K;
+      top[i + (size_t)k * ldt] = M[i + (size_t)k * ldm];
+    }
     return;
   }
-  const int r0 = bk + (blockIdx.x - 1) * rt;
-  const int rows = min(rt, mk - r0);
-  for (int k = 0; k < bk; ++k)
-    for (int i = tid; i <= k; i += kFinThreads) U[uoff(i) + (k - i)] = lu11[i + (size_t)k * ldl];
-  for (int i = tid; i < bk; i += kFinThreads) rd[i] = 1.0 / lu11[i + (size_t)i * ldl];
-  for (int k = 0; k < bk; ++k)
-    for (int i = tid; i < rows; i += kFinThreads) T[i + (size_t)k * rt] = P[r0 + i + (size_t)k * lda];
-  __syncthreads();
-  // thread (r, g): row r, columns k = j + 1 + g (mod ng); rt <= kFinThreads
-  const int ng = kFinThreads / rt;
-  const int g = tid / rt, r = tid - g * rt;
-  for (int j = 0; j < bk; ++j) {
-    for (int i = tid; i < rows; i += kFinThreads) T[i + (size_t)j * rt] *= rd[j];
-    __syncthreads();
-    if (g < ng && r < rows) {
-      const double x = T[r + (size_t)j * rt];
-      const double *uj = U + uoff(j) - j;  // uj[k] = U(j, k)
-      for (int k = j + 1 + g; k < bk; k += ng) T[r + (size_t)k * rt] = fma(-x, uj[k], T[r + (size_t)k * rt]);
-    }
-    __syncthreads();
+  double *C = tsm, *rd = tsm + (size_t)K * TPR * CPT;
+  // triangle row j: elements k > j, zero elsewhere; coalesced along M's columns
+  for (int idx = tid; idx < K * K; idx += kTriThreads) {
+    const int i = idx % K, q = idx / K;  // M(i, q)
+    const int j = ROWS ? i : q, k = ROWS ? q : i;
+    const double v = M[i + (size_t)q * ldm];
+    const int kk = k / TPR;
+    C[(size_t)j * (TPR * CPT) + 4 * TPR * (kk >> 2) + 4 * (k % TPR) + (kk & 3)] = k > j ? v : 0.0;
+    if (ROWS && k == j) rd[j] = 1.0 / v;
   }
-  for (int k = 0; k < bk; ++k)
-    for (int i = tid; i < rows; i += kFinThreads) P[r0 + i + (size_t)k * lda] = T[i + (size_t)k * rt];
-}
-
-// ---------------------------------------------------------------------------
-// U12 = L11^-1 A12 (unit lower), one CTA per tile of ct columns.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) trsm_u12_kernel(int bk, int nt, const double *L, int ldl,
-                                                       double *A, int lda, int ct, const int *skip) {
-  extern __shared__ __align__(16) double usm[];
-  if (skip && *skip) return;
-  double *Ls = usm;                   // bk x bk, ld bk
-  double *T = Ls + (size_t)bk * bk;   // bk x ct, ld bk
-  const int tid = threadIdx.x;
-  const int c0 = blockIdx.x * ct;
-  const int cols = min(ct, nt - c0);
-  for (int k = 0; k < bk; ++k)
-    for (int i = tid; i < bk; i += 256) Ls[i + (size_t)k * bk] = (i > k) ? L[i + (size_t)k * ldl] : 0.0;
-  for (int c = 0; c < cols; ++c)
-    for (int i = tid; i < bk; i += 256) T[i + (size_t)c * bk] = A[i + (size_t)(c0 + c) * lda];
-  __syncthreads();
-  // thread (row group, column): rows i > j updated after row j is final
-  for (int j = 0; j < bk - 1; ++j) {
-    const int nr = bk - j - 1;
-    for (int idx = tid; idx < nr * cols; idx += 256) {
-      int c = idx / nr, i = j + 1 + (idx - (idx / nr) * nr);
-      T[i + (size_t)c * bk] = fma(-Ls[i + (size_t)j * bk], T[j + (size_t)c * bk], T[i + (size_t)c * bk]);
-    }
-    __syncthreads();
+  TriSolve<TPR, CPT, ROWS> t;
+  t.C = C;
+  t.rd = rd;
+  t.K = K;
+  t.sub = tid % TPR;
+  const int lv = tid / TPR, v = blockIdx.x * vb + lv;
+  const bool live = lv < vb && v < nv;
+  double *x = X + (ROWS ? (size_t)v : (size_t)v * ldx);
+  const size_t step = ROWS ? (size_t)ldx : 1;
+#pragma unroll
+  for (int k = 0; k < CPT; ++k) {
+    const int e = k * TPR + t.sub;
+    t.a[k] = (live && e < K) ? x[(size_t)e * step] : 0.0;
   }
-  for (int c = 0; c < cols; ++c)
-    for (int i = tid; i < bk; i += 256) A[i + (size_t)(c0 + c) * lda] = T[i + (size_t)c * bk];
+  // registers beyond K read what the rows hold there: keep it finite
+  for (int idx = tid; idx < K * (TPR * CPT - K); idx += kTriThreads) {
+    const int j = idx % K, k = K + idx / K, kk = k / TPR;
+    C[(size_t)j * (TPR * CPT) + 4 * TPR * (kk >> 2) + 4 * (k % TPR) + (kk & 3)] = 0.0;
+  }
+  __syncthreads();
+  if ((tid & ~31) / TPR >= vb) return;  // a warp without vectors
+  int j = 0, nb = ((K + TPR - 1) / TPR + 3) / 4;
+#pragma unroll 1
+  while (t.template group<0>(j, nb, x, step, live) && t.template group<1>(j, nb, x, step, live) &&
+         t.template group<2>(j, nb, x, step, live) && t.template group<3>(j, nb, x, step, live)) {
+#pragma unroll
+    for (int k = 0; k + 4 < CPT; ++k) t.a[k] = t.a[k + 4];
+    --nb;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -643,53 +674,54 @@ cudaError_t laswp_apply(int ncols, double *A, int lda, int row0, const LuPanelWs
   return cudaGetLastError();
 }
 
-cudaError_t lu_panel_finish(int mk, int bk, double *P, int lda, const LuPanelWs &ws,
-                            cudaStream_t st, const int *skip) {
+template <int TPR, int CPT, bool ROWS>
+static cudaError_t launch_tri1(int nv, int K, const double *M, int ldm, double *X, int ldx, int vb, double *top, int ldt,
+                               cudaStream_t st, const int *skip) {
   static std::atomic<unsigned long long> init{0};
   cudaError_t e = once_per_device(init, [] {
-    return cudaFuncSetAttribute(lu_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    return cudaFuncSetAttribute(tri_panel_kernel<TPR, CPT, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                TPR * CPT * (TPR * CPT + 1) * 8);
   });
   if (e != cudaSuccess) return e;
-  // row tiles sized so that the rows below the panel's top fill one wave
-  // of one CTA per SM where they can (shared memory: packed U plus the tile)
-  int sms = 0;
-  if ((e = device_sm_count(&sms)) != cudaSuccess) return e;
-  const int below = mk - bk;
-  const size_t ubytes = ((size_t)bk * (bk + 1) / 2 + bk) * 8;
-  int rtmax = (int)((200 * 1024 - ubytes) / ((size_t)bk * 8));
-  if (rtmax > kFinThreads / 2) rtmax = kFinThreads / 2;  // at least two threads per row
-  int rt = below > 0 ? (below + sms - 1) / sms : 1;
-  rt = (rt + 7) / 8 * 8;
-  if (rt < 32) rt = 32;
-  if (rt > rtmax) rt = rtmax;
-  size_t smem = ubytes + (size_t)rt * bk * 8;
-  int nblk = 1 + (below > 0 ? (below + rt - 1) / rt : 0);
-  ProfScope ps(kClsLuFinish, st, (double)(below > 0 ? below : 0) * bk * bk);
-  lu_finish_kernel<<<nblk, kFinThreads, smem, st>>>(mk, bk, P, lda, ws.lu11, bk, rt, skip);
+  const size_t smem = (size_t)K * (TPR * CPT + 1) * 8;
+  const int grid = (nv + vb - 1) / vb + (ROWS ? 1 : 0);
+  tri_panel_kernel<TPR, CPT, ROWS><<<grid, kTriThreads, smem, st>>>(nv, K, M, ldm, X, ldx, vb, top, ldt, skip);
   return cudaGetLastError();
+}
+
+// Four threads per vector when the vectors fill the SMs that way, else 16 (the
+// chain of multiply-adds per thread is shorter and more SMs take part).
+template <bool ROWS>
+static cudaError_t launch_tri(int nv, int K, const double *M, int ldm, double *X, int ldx, double *top, int ldt,
+                              cudaStream_t st, const int *skip) {
+  int sms = 0;
+  cudaError_t e = device_sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const bool few = nv <= sms * (kTriThreads / 16);
+  const int most = kTriThreads / (few ? 16 : 4);
+  int vb = (nv + sms - 1) / sms;
+  const int unit = few ? 2 : 8;  // vectors of a warp
+  vb = (vb + unit - 1) / unit * unit;
+  vb = vb < 1 ? unit : vb > most ? most : vb;
+  if (K <= 64)
+    return few ? launch_tri1<16, 4, ROWS>(nv, K, M, ldm, X, ldx, vb, top, ldt, st, skip)
+               : launch_tri1<4, 16, ROWS>(nv, K, M, ldm, X, ldx, vb, top, ldt, st, skip);
+  return few ? launch_tri1<16, 8, ROWS>(nv, K, M, ldm, X, ldx, vb, top, ldt, st, skip)
+             : launch_tri1<4, 32, ROWS>(nv, K, M, ldm, X, ldx, vb, top, ldt, st, skip);
+}
+
+cudaError_t lu_panel_finish(int mk, int bk, double *P, int lda, const LuPanelWs &ws,
+                            cudaStream_t st, const int *skip) {
+  const int below = mk - bk > 0 ? mk - bk : 0;
+  ProfScope ps(kClsLuFinish, st, (double)below * bk * bk);
+  return launch_tri<true>(below, bk, ws.lu11, bk, P + bk, lda, P, lda, st, skip);
 }
 
 cudaError_t trsm_u12(int bk, int nt, const double *L11, int ldl, double *A12, int lda,
                      cudaStream_t st, const int *skip) {
-  static std::atomic<unsigned long long> init{0};
-  cudaError_t e = once_per_device(init, [] {
-    return cudaFuncSetAttribute(trsm_u12_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-  });
-  if (e != cudaSuccess) return e;
   if (nt <= 0 || bk <= 1) return cudaSuccess;
-  // column tiles: as many CTAs as SMs where the columns allow (the look-ahead
-  // solve of the next panel's b columns is on the panel chain), at most
-  // 8192 / bk columns each
-  int sms = 0;
-  if ((e = device_sm_count(&sms)) != cudaSuccess) return e;
-  int ct = (nt + sms - 1) / sms;
-  const int ctmax = 8192 / bk < 128 ? 8192 / bk : 128;
-  if (ct > ctmax) ct = ctmax;
-  if (ct < 1) ct = 1;
-  size_t smem = ((size_t)bk * bk + (size_t)bk * ct) * 8;
   ProfScope ps(kClsTrsmU12, st, (double)bk * bk * nt);
-  trsm_u12_kernel<<<(nt + ct - 1) / ct, 256, smem, st>>>(bk, nt, L11, ldl, A12, lda, ct, skip);
-  return cudaGetLastError();
+  return launch_tri<false>(nt, bk, L11, ldl, A12, lda, nullptr, 0, st, skip);
 }
 
 }  // namespace cagb
