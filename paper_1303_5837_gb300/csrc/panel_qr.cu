@@ -665,6 +665,9 @@ __global__ void __launch_bounds__(kApThreads, 1) tree_apply_kernel(ApplyArgs a) 
 //   phase 3: thread (row i = tid % 32, k-slice q = tid / 32 of 16 reflectors)
 //            sums Y(i, k) W(k, :) over its slice; the 8 slices are added in
 //            shared memory and subtracted from C.
+// A node may be spread over the G CTAs of a cluster: each takes every G-th
+// chunk of rows in phases 1 and 3, the partial W are added in rank order
+// through distributed shared memory, and every CTA forms T^T W itself.
 // ---------------------------------------------------------------------------
 constexpr int kNcChunk = 32;
 
@@ -678,7 +681,9 @@ __global__ void __launch_bounds__(kApThreads, 2) tree_apply_narrow_kernel(ApplyA
   double *Ws = Cs + kNcChunk * NC;         // 128 x NC
   double *red = Ws + 128 * NC;             // 8 x kNcChunk x NC (phase 3), 128 x NC (phase 1)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int node = blockIdx.x;
+  cg::cluster_group cl = cg::this_cluster();
+  const int G = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int node = blockIdx.x / G;
   const int c0 = blockIdx.y * NC;
   const int ncl = min(NC, a.ncols - c0);
 
@@ -688,7 +693,7 @@ __global__ void __launch_bounds__(kApThreads, 2) tree_apply_narrow_kernel(ApplyA
     lrow0 = node * a.leaf_rows;
     lrows = min(a.leaf_rows, a.mk - lrow0);
     kk = min(lrows, bk);
-    if (blockIdx.y == 0 && tid == 0) {
+    if (blockIdx.y == 0 && tid == 0 && rank == 0) {
       a.top_out[node] = lrow0;
       a.c_out[node] = kk;
     }
@@ -697,7 +702,7 @@ __global__ void __launch_bounds__(kApThreads, 2) tree_apply_narrow_kernel(ApplyA
     int R = 0;
     for (int ch = 0; ch < cnt; ++ch) R += a.c_in[start + ch];
     kk = min(R, bk);
-    if (blockIdx.y == 0 && tid == 0) {
+    if (blockIdx.y == 0 && tid == 0 && rank == 0) {
       a.top_out[node] = a.top_in[start];
       a.c_out[node] = (cnt == 1) ? a.c_in[start] : kk;
     }
@@ -739,11 +744,12 @@ __global__ void __launch_bounds__(kApThreads, 2) tree_apply_narrow_kernel(ApplyA
   double acc[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) acc[c] = 0.0;
+  int chunk = 0;
   for (int sg = 0; sg < nseg; ++sg) {
     int srow, srows, type;
     segment(sg, srow, srows, type);
     if (type == 1) {  // identity block: W(k, :) += C(k, :)
-      if (h1 == 0 && k1 < srows) {
+      if (rank == 0 && h1 == 0 && k1 < srows) {
 #pragma unroll
         for (int c = 0; c < NC; ++c)
           if (c < ncl) acc[c] += a.C[srow + k1 + (size_t)(c0 + c) * a.ldc];
@@ -751,6 +757,7 @@ __global__ void __launch_bounds__(kApThreads, 2) tree_apply_narrow_kernel(ApplyA
       continue;
     }
     for (int r0 = 0; r0 < srows; r0 += kNcChunk) {
+      if (chunk++ % G != rank) continue;
       const int nr = min(kNcChunk, srows - r0);
       __syncthreads();
       stage_y(srow, type, r0, nr);
@@ -785,6 +792,24 @@ __global__ void __launch_bounds__(kApThreads, 2) tree_apply_narrow_kernel(ApplyA
     for (int c = 0; c < NC; ++c) Ws[k1 * NC + c] = acc[c] + red[k1 * NC + c];
   }
   __syncthreads();
+  if (G > 1) {  // the sum of the cluster's partial W, in rank order
+    cl.sync();
+    double w[(128 * NC + kApThreads - 1) / kApThreads];
+#pragma unroll
+    for (int u = 0; u < (128 * NC + kApThreads - 1) / kApThreads; ++u) {
+      const int e = tid + u * kApThreads;
+      w[u] = 0.0;
+      if (e < 128 * NC)
+        for (int r = 0; r < G; ++r) w[u] += *cl.map_shared_rank(Ws + e, r);
+    }
+    cl.sync();  // every partial has been read
+#pragma unroll
+    for (int u = 0; u < (128 * NC + kApThreads - 1) / kApThreads; ++u) {
+      const int e = tid + u * kApThreads;
+      if (e < 128 * NC) Ws[e] = w[u];
+    }
+    __syncthreads();
+  }
 
   // ---- phase 2: W <- T^T W (T upper triangular, kk x kk) ------------------
   double s[NC];
@@ -807,17 +832,20 @@ __global__ void __launch_bounds__(kApThreads, 2) tree_apply_narrow_kernel(ApplyA
 
   // ---- phase 3: C -= Y W ----------------------------------------------------
   const int kq = 16 * warp;  // this warp's 16 reflectors
+  chunk = 0;
   for (int sg = 0; sg < nseg; ++sg) {
     int srow, srows, type;
     segment(sg, srow, srows, type);
     if (type == 1) {
-      for (int idx = tid; idx < srows * ncl; idx += kApThreads) {
-        const int i = idx % srows, c = idx / srows;
-        a.C[srow + i + (size_t)(c0 + c) * a.ldc] -= Ws[i * NC + c];
-      }
+      if (rank == 0)
+        for (int idx = tid; idx < srows * ncl; idx += kApThreads) {
+          const int i = idx % srows, c = idx / srows;
+          a.C[srow + i + (size_t)(c0 + c) * a.ldc] -= Ws[i * NC + c];
+        }
       continue;
     }
     for (int r0 = 0; r0 < srows; r0 += kNcChunk) {
+      if (chunk++ % G != rank) continue;
       const int nr = min(kNcChunk, srows - r0);
       __syncthreads();
       stage_y(srow, type, r0, nr);
@@ -1007,22 +1035,39 @@ cudaError_t tree_apply_qt(int mk, int bk, int b, const double *P, int lda, int l
   const int ntiles = (ncols + kCt - 1) / kCt;
   // narrow kernel for a few columns, or when the 32-column tiles of the leaf
   // update would leave SMs without a CTA
-  const int nc = ncols <= 1 ? 1 : ncols <= 2 ? 2 : ncols <= 4 ? 4 : 8;
   const bool narrow = ncols <= 8 || (long long)plan.nleaves * ntiles < sms;
-  const int gy = narrow ? (ncols + nc - 1) / nc : ntiles;
-  const size_t nsmem = narrow_smem_bytes(bk, nc);
-  auto launch = [&](int gx) {
-    const dim3 grid(gx, gy);
-    if (!narrow)
-      tree_apply_kernel<<<grid, kApThreads, smem, st>>>(a);
-    else if (nc == 1)
-      tree_apply_narrow_kernel<1><<<grid, kApThreads, nsmem, st>>>(a);
-    else if (nc == 2)
-      tree_apply_narrow_kernel<2><<<grid, kApThreads, nsmem, st>>>(a);
-    else if (nc == 4)
-      tree_apply_narrow_kernel<4><<<grid, kApThreads, nsmem, st>>>(a);
-    else
-      tree_apply_narrow_kernel<8><<<grid, kApThreads, nsmem, st>>>(a);
+  // a launch over gx nodes of at most `rows` rows
+  auto launch = [&](int gx, int rows) -> cudaError_t {
+    if (!narrow) {
+      tree_apply_kernel<<<dim3(gx, ntiles), kApThreads, smem, st>>>(a);
+      return cudaGetLastError();
+    }
+    // as few columns per CTA as keep the launch within two CTAs per SM (the
+    // look-ahead update of CAQR 1024 x 1024, 8 nodes x 64 columns: 73 us a
+    // launch with 8 columns, 43 now), then a cluster per node where SMs are
+    // still left (Q^T b through 1024-row leaves, 6 nodes x 1 column: 231 us,
+    // 45 now)
+    int nc = ncols <= 1 ? 1 : ncols <= 2 ? 2 : ncols <= 4 ? 4 : 8;
+    while (nc > 1 && (long long)gx * ((ncols + nc / 2 - 1) / (nc / 2)) <= 2 * sms) nc /= 2;
+    const int gy = (ncols + nc - 1) / nc;
+    int G = 1;
+    while (G < 8 && (long long)gx * gy * G * 2 <= sms && rows > kNcChunk * G) G *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(gx * G, gy);
+    cfg.blockDim = dim3(kApThreads);
+    cfg.dynamicSmemBytes = narrow_smem_bytes(bk, nc);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = G;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return nc == 1   ? cudaLaunchKernelEx(&cfg, tree_apply_narrow_kernel<1>, a)
+           : nc == 2 ? cudaLaunchKernelEx(&cfg, tree_apply_narrow_kernel<2>, a)
+           : nc == 4 ? cudaLaunchKernelEx(&cfg, tree_apply_narrow_kernel<4>, a)
+                     : cudaLaunchKernelEx(&cfg, tree_apply_narrow_kernel<8>, a);
   };
   a.is_leaf = 1;
   a.top_out = ws.top[0];
@@ -1037,9 +1082,8 @@ cudaError_t tree_apply_qt(int mk, int bk, int b, const double *P, int lda, int l
       f += (4.0 * (r * k - k * (k - 1) / 2.0) + k * (k + 1)) * ncols;
     }
     ProfScope ps(narrow ? kClsTreeNarrow : kClsTreeApply, st, f);
-    launch(plan.nleaves);
+    e = launch(plan.nleaves, leaf_rows < mk ? leaf_rows : mk);
   }
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   int buf = 0;
   for (int r = 0; r < plan.nrounds; ++r) {
@@ -1062,9 +1106,8 @@ cudaError_t tree_apply_qt(int mk, int bk, int b, const double *P, int lda, int l
         if (cnt >= 2) f += (4.0 * (cnt - 1) * kb2 * (kb2 + 1) / 2.0 + kb2 * (kb2 + 1) + 2.0 * kb2) * ncols;
       }
       ProfScope ps(narrow ? kClsTreeNarrow : kClsTreeApply, st, f);
-      launch(plan.r[r].n_out);
+      e = launch(plan.r[r].n_out, (rd.max_cnt - 1) * bk);
     }
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     buf ^= 1;
   }
