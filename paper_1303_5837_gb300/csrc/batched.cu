@@ -17,6 +17,7 @@
 
 #include "ca_internal.cuh"
 #include "device_once.cuh"
+#include "qr_node_reg.cuh"
 
 namespace cagb {
 namespace {
@@ -167,6 +168,177 @@ __device__ int node_gepp(T *tile, int ld, int rows, int bk, int *lab, Fixed<T> &
     __syncthreads();
   }
   return kmax;
+}
+
+// ---------------------------------------------------------------------------
+// The same node in registers, for up to 512 rows and 32 columns: a thread
+// holds two rows (tid, tid + 256) with every column, rows never move (each
+// carries its position after the interchanges so far, as in panel_lu_reg.cu),
+// and a column takes two barriers: the warps' best rows, then the pivot row
+// and its reciprocal.  Loads the rows F.prow[0..rows) of the panel; on return
+// F.prow[0..kmax) are the chosen labels in pivot order and, at the root, lu11
+// (ld b) holds their L \ U.  R: shared scratch.
+// ---------------------------------------------------------------------------
+constexpr int kGeppRows = 2 * kBT, kGeppCols = 32;
+constexpr int kGeppU = kGeppCols + 8;  // a published row: reciprocal, pad, then the columns
+
+__device__ __forceinline__ float recip_of(float v) { return 1.0f / v; }
+__device__ __noinline__ double recip_lib(double v) { return 1.0 / v; }
+__device__ __forceinline__ double recip_of(double v) {
+  const double r = recip_exact_or_zero(v);
+  return __double_as_longlong(r) != 0 ? r : recip_lib(v);
+}
+
+template <class T>
+struct GeppNode {
+  T a[2][kGeppCols];
+  int pos[2];
+  T *u;          // [2][kGeppU], by column parity
+  ArgMax *best;  // [2][kBW]
+  T *keep;       // root: this thread's place for finished columns of its rows (or null), rows kBT ldk apart
+  int ldk;
+  int kmax, nb;  // nb: blocks of 4 columns left
+  unsigned long long key;
+  int p;
+
+  __device__ __forceinline__ void post(int j, unsigned long long k0, unsigned long long k1) {
+    ArgMax m{k0, k0 != 0ull ? pos[0] : INT_MAX};
+    m = argmax_better(m, ArgMax{k1, k1 != 0ull ? pos[1] : INT_MAX});
+    m = warp_argmax(m);
+    if ((threadIdx.x & 31) == 0) best[(j & 1) * kBW + (threadIdx.x >> 5)] = m;
+  }
+  __device__ __forceinline__ void take(int j) {
+    ArgMax m{0ull, INT_MAX};
+#pragma unroll
+    for (int w = 0; w < kBW; ++w) m = argmax_better(m, best[(j & 1) * kBW + w]);
+    key = m.key;
+    p = m.pos;
+  }
+  // column j = 4 (blocks done) + Q; false after the last one
+  template <int Q>
+  __device__ __forceinline__ bool column(int j, Fixed<T> &F, bool root, int kb) {
+    T *uj = u + (j & 1) * kGeppU;
+    const bool zero = key == 0ull;
+    if (!zero) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+        if (pos[r] == p) {
+#pragma unroll
+          for (int k = 0; k < kGeppCols; ++k) {
+            if (k >= 4 * nb) break;
+            uj[8 + k] = a[r][k];
+          }
+          uj[0] = recip_of(a[r][Q]);
+        }
+    }
+    __syncthreads();
+    if (zero && root && threadIdx.x == 0 && F.info0 == 0) F.info0 = kb + j + 1;
+    unsigned long long kn[2] = {0ull, 0ull};
+    const bool more = j + 1 < kmax;
+    T l[2];
+    bool act[2];
+    const T rinv = uj[0];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      if (!zero) pos[r] = pos[r] == p ? j : pos[r] == j ? p : pos[r];
+      act[r] = pos[r] > j && !zero;
+      l[r] = T(0);
+      if (act[r]) {
+        l[r] = a[r][Q] * rinv;
+        a[r][Q] = l[r];
+        a[r][Q + 1] = fma(-l[r], uj[8 + Q + 1], a[r][Q + 1]);
+      }
+      if (pos[r] > j) kn[r] = Num<T>::key(a[r][Q + 1]);
+    }
+    if (more) post(j + 1, kn[0], kn[1]);
+#pragma unroll
+    for (int c = 0; c < kGeppCols / 4; ++c) {
+      if (c >= nb) break;
+#pragma unroll
+      for (int k = 4 * c; k < 4 * c + 4; ++k) {
+        if (k < Q + 2) continue;
+        const T w = uj[8 + k];
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+          if (act[r]) a[r][k] = fma(-l[r], w, a[r][k]);
+      }
+    }
+    if (keep) {
+      keep[Q] = a[0][Q];
+      keep[(size_t)kBT * ldk + Q] = a[1][Q];
+    }
+    if (!more) return false;
+    __syncthreads();
+    take(j + 1);
+    return true;
+  }
+};
+
+template <class T>
+__device__ __noinline__ int node_gepp_reg(const T *P, int lda, int rows, int bk, Fixed<T> &F, bool root, int kb, T *R,
+                                          T *lu11, int b) {
+  const int tid = threadIdx.x;
+  GeppNode<T> g;
+  g.u = R;
+  g.best = reinterpret_cast<ArgMax *>(R + 2 * kGeppU);
+  T *keep = reinterpret_cast<T *>(g.best + 2 * kBW);
+  g.ldk = (bk + 3) / 4 * 4 + 1;  // odd: rows of a warp in distinct banks
+  g.keep = root ? keep + (size_t)tid * g.ldk : nullptr;
+  g.kmax = min(rows, bk);
+  g.nb = (bk + 3) / 4;
+  int lab[2];
+  bool bad = false;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int q = tid + r * kBT;
+    lab[r] = q < rows ? F.prow[q] : -1;
+    g.pos[r] = q < rows ? q : -1;
+#pragma unroll
+    for (int k = 0; k < kGeppCols; ++k) {
+      T v = T(0);
+      if (lab[r] >= 0 && k < bk) v = P[lab[r] + (size_t)k * lda];
+      bad |= Num<T>::bad(v);
+      g.a[r][k] = v;
+    }
+  }
+  if (bad) atomicOr(&F.status, CA_STATUS_NONFINITE);
+  // (also: every read of F.prow and of R's earlier contents is done)
+  g.post(0, g.pos[0] >= 0 ? Num<T>::key(g.a[0][0]) : 0ull, g.pos[1] >= 0 ? Num<T>::key(g.a[1][0]) : 0ull);
+  __syncthreads();
+  g.take(0);
+  int j = 0;
+#pragma unroll 1
+  while (true) {
+    if (!g.template column<0>(j, F, root, kb) || !g.template column<1>(j + 1, F, root, kb) ||
+        !g.template column<2>(j + 2, F, root, kb) || !g.template column<3>(j + 3, F, root, kb))
+      break;
+    j += 4;
+    --g.nb;
+    if (g.keep) g.keep += 4;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int k = 0; k + 4 < kGeppCols; ++k) g.a[r][k] = g.a[r][k + 4];
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+    if (g.pos[r] >= 0 && g.pos[r] < g.kmax) {
+      F.prow[g.pos[r]] = lab[r];
+      if (root) {
+        const T *kr = keep + (size_t)(tid + r * kBT) * g.ldk;
+        for (int k = 0; k < bk; ++k) lu11[g.pos[r] + (size_t)k * b] = kr[k];
+      }
+    }
+  __syncthreads();
+  return g.kmax;
+}
+
+// Whether a node's rows fit node_gepp_reg (with room for its scratch).
+template <class T>
+__device__ __forceinline__ bool gepp_reg_fits(int rows, int bk, const ca_tree_t &tr, bool root, int region_elems) {
+  const int keep = root ? kGeppRows * ((bk + 3) / 4 * 4 + 1) : 0;
+  return tr.op_depth == 0 && rows <= kGeppRows && bk <= kGeppCols &&
+         2 * kGeppU + (int)(2 * kBW * sizeof(ArgMax) / sizeof(T)) + keep <= region_elems;
 }
 
 // ---------------------------------------------------------------------------
@@ -401,11 +573,17 @@ __device__ void cta_calu(const ca_batch_item_t &it, Fixed<T> &F, T *R, int regio
       const int r0 = j * L, rows = min(L, mk - r0), ld = odd_ld(rows);
       for (int p = tid; p < rows; p += kBT) F.prow[p] = r0 + p;
       __syncthreads();
-      load_rows(P, lda, rows, bk, R, ld, F, false);
-      const int km = node_op(R, ld, rows, bk, F, nrounds == 0, kb, it.tree, wsi);
+      const bool regs = gepp_reg_fits<T>(rows, bk, it.tree, nrounds == 0, region_elems);
+      int km;
+      if (regs) {
+        km = node_gepp_reg<T>(P, lda, rows, bk, F, nrounds == 0, kb, R, lu11, b);
+      } else {
+        load_rows(P, lda, rows, bk, R, ld, F, false);
+        km = node_op(R, ld, rows, bk, F, nrounds == 0, kb, it.tree, wsi);
+      }
       for (int p = tid; p < km; p += kBT) cand[0][(size_t)j * b + p] = F.prow[p];
       if (tid == 0) ncand[0][j] = km;
-      if (nrounds == 0)
+      if (nrounds == 0 && !regs)
         for (int k = warp; k < bk; k += kBW)
           for (int p = lane; p < bk; p += 32) lu11[p + (size_t)k * b] = R[p + (size_t)k * ld];
       __syncthreads();
@@ -436,11 +614,17 @@ __device__ void cta_calu(const ca_batch_item_t &it, Fixed<T> &F, T *R, int regio
         }
         __syncthreads();
         const int ld = odd_ld(rows);
-        load_rows(P, lda, rows, bk, R, ld, F, false);
-        const int km = node_op(R, ld, rows, bk, F, last, kb, it.tree, wsi);
+        const bool regs = gepp_reg_fits<T>(rows, bk, it.tree, last, region_elems);
+        int km;
+        if (regs) {
+          km = node_gepp_reg<T>(P, lda, rows, bk, F, last, kb, R, lu11, b);
+        } else {
+          load_rows(P, lda, rows, bk, R, ld, F, false);
+          km = node_op(R, ld, rows, bk, F, last, kb, it.tree, wsi);
+        }
         for (int p = tid; p < km; p += kBT) cout[(size_t)o * b + p] = F.prow[p];
         if (tid == 0) nout[o] = km;
-        if (last)
+        if (last && !regs)
           for (int k = warp; k < bk; k += kBW)
             for (int p = lane; p < bk; p += 32) lu11[p + (size_t)k * b] = R[p + (size_t)k * ld];
         __syncthreads();
@@ -804,6 +988,93 @@ __device__ int merge_rows(const int *top, const int *c, int start, int cnt, Fixe
   return rows;
 }
 
+// The same for a node in registers: the other children's rows in the order of
+// their index within the child where all have one height (NodeRows).
+template <class T>
+__device__ NodeRows<true> merge_rows_reg(const int *top, const int *c, int start, int cnt, int rows, int kmax,
+                                         Fixed<T> &F) {
+  NodeRows<true> nr;
+  nr.R = rows;
+  nr.reord = nr.beg = nr.c0 = nr.nk = nr.h = 0;
+  const int c0 = c[start], h = c[start + 1];
+  bool same = true;
+  for (int ch = 2; ch < cnt; ++ch) same &= c[start + ch] == h;
+  if (!same || c0 < kmax) {
+    merge_rows(top, c, start, cnt, F);
+    return nr;
+  }
+  nr.reord = 1;
+  nr.c0 = c0;
+  nr.nk = cnt - 1;
+  nr.h = h;
+  nr.beg = c0 >> 4;
+  for (int p = threadIdx.x; p < rows; p += kBT) {
+    const int t = p < c0 ? p : (p - c0) / nr.nk, ch = p < c0 ? 0 : 1 + (p - c0) % nr.nk;
+    F.prow[p] = top[start + ch] + t;
+    F.fz[p] = t;
+  }
+  __syncthreads();
+  return nr;
+}
+
+// A QR node in registers (qr_node_reg.cuh): loads the rows F.prow[0..rows) of
+// the panel (zero left of F.fz in a merge), factors them, writes the rows and
+// T back.  nr: the order of the rows (a merge's may be reordered).  The
+// shared-memory tile it replaces (node_qr) takes four barriers and a serial
+// reflector per column and three shared-memory accesses per multiply-add.
+template <class T, int TC, int TS>
+__device__ __noinline__ int node_qr_reg(T *P, int lda, int rows, int bk, const NodeRows<true> &nr, bool use_fz,
+                                        Fixed<T> &F, T *Tg, int b, T *R) {
+  RegSmem<T, TC, TS> &sm = *reinterpret_cast<RegSmem<T, TC, TS> *>(R);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int rg = lane & 15, cg = 2 * (tid >> 5) + (lane >> 4);
+  const int kmax = min(rows, bk);
+  T A[TS][TC];
+  bool bad = false;
+#pragma unroll
+  for (int s = 0; s < TS; ++s) {
+    const int p = rg + 16 * s;
+    const int prow = p < rows ? F.prow[p] : -1, fz = (use_fz && p < rows) ? F.fz[p] : 0;
+#pragma unroll
+    for (int t = 0; t < TC; ++t) {
+      const int q = cg + 16 * t;
+      T v = T(0);
+      if (prow >= 0 && q < bk && q >= fz) v = P[prow + (size_t)q * lda];
+      bad |= Num<T>::bad(v);
+      A[s][t] = v;
+    }
+  }
+  if (bad) atomicOr(&F.status, CA_STATUS_NONFINITE);
+  qr_node<T, TC, TS, true>(A, nr, sm, kmax);
+  for (int idx = tid; idx < b * b; idx += kBT) {
+    const int i = idx % b, jj = idx / b;
+    T v = T(0);
+    if (jj < kmax && i <= jj) v = (i == jj) ? sm.tau[jj] : sm.T[jj * (jj - 1) / 2 + i];
+    Tg[idx] = v;
+  }
+#pragma unroll
+  for (int s = 0; s < TS; ++s) {
+    const int p = rg + 16 * s;
+    const int prow = p < rows ? F.prow[p] : -1, fz = (use_fz && p < rows) ? F.fz[p] : 0;
+#pragma unroll
+    for (int t = 0; t < TC; ++t) {
+      const int q = cg + 16 * t;
+      if (prow >= 0 && q < bk && q >= fz) P[prow + (size_t)q * lda] = A[s][t];
+    }
+  }
+  return kmax;
+}
+
+// Nodes of up to 512 rows and 32 columns, or 256 rows and 64 columns.
+__device__ __forceinline__ bool qr_reg_fits(int rows, int bk) { return bk <= 32 ? rows <= 512 : bk <= 64 && rows <= 256; }
+
+template <class T>
+__device__ __forceinline__ int node_qr_regs(T *P, int lda, int rows, int bk, const NodeRows<true> &nr, bool use_fz,
+                                            Fixed<T> &F, T *Tg, int b, T *R) {
+  return bk > 32 ? node_qr_reg<T, 4, 16>(P, lda, rows, bk, nr, use_fz, F, Tg, b, R)
+                 : node_qr_reg<T, 2, 32>(P, lda, rows, bk, nr, use_fz, F, Tg, b, R);
+}
+
 // C <- Q_node^T C for the node rows F.prow[0..rows) (leaf: Y unit lower
 // trapezoid stored in those rows; merge: identity on the first child's rows,
 // stored upper trapezoids on the others), nref <= TK reflectors, T block Tg.
@@ -986,10 +1257,17 @@ __device__ void cta_caqr(const ca_batch_item_t &it, Fixed<T> &F, T *R, int regio
       const int r0 = j * L, rows = min(L, mk - r0), ld = odd_ld(rows);
       for (int p = tid; p < rows; p += kBT) F.prow[p] = r0 + p;
       __syncthreads();
-      load_rows(P, lda, rows, bk, R, ld, F, false);
-      const int km = node_qr(R, ld, rows, bk, F, false, Tp + (size_t)j * b * b, b, region_elems);
-      for (int k = warp; k < bk; k += kBW)
-        for (int p = lane; p < rows; p += 32) P[r0 + p + (size_t)k * lda] = R[p + (size_t)k * ld];
+      int km;
+      if (qr_reg_fits(rows, bk)) {
+        NodeRows<true> nr = {};
+        nr.R = rows;  // every row block takes part
+        km = node_qr_regs(P, lda, rows, bk, nr, false, F, Tp + (size_t)j * b * b, b, R);
+      } else {
+        load_rows(P, lda, rows, bk, R, ld, F, false);
+        km = node_qr(R, ld, rows, bk, F, false, Tp + (size_t)j * b * b, b, region_elems);
+        for (int k = warp; k < bk; k += kBW)
+          for (int p = lane; p < rows; p += 32) P[r0 + p + (size_t)k * lda] = R[p + (size_t)k * ld];
+      }
       if (tid == 0) {
         top[0][j] = r0;
         cc[0][j] = km;
@@ -1011,13 +1289,22 @@ __device__ void cta_caqr(const ca_batch_item_t &it, Fixed<T> &F, T *R, int regio
           __syncthreads();
           continue;
         }
-        const int rows = merge_rows(top[buf], cc[buf], start, cnt, F);
-        const int ld = odd_ld(rows);
-        load_rows(P, lda, rows, bk, R, ld, F, true);
-        const int km = node_qr(R, ld, rows, bk, F, true, Tp + (size_t)(nl + midx) * b * b, b, region_elems);
-        for (int k = warp; k < bk; k += kBW)
-          for (int p = lane; p < rows; p += 32)
-            if (k >= F.fz[p]) P[F.prow[p] + (size_t)k * lda] = R[p + (size_t)k * ld];
+        int rows = 0;
+        for (int ch = 0; ch < cnt; ++ch) rows += cc[buf][start + ch];
+        T *Tg = Tp + (size_t)(nl + midx) * b * b;
+        int km;
+        if (qr_reg_fits(rows, bk)) {
+          const NodeRows<true> nr = merge_rows_reg(top[buf], cc[buf], start, cnt, rows, min(rows, bk), F);
+          km = node_qr_regs(P, lda, rows, bk, nr, true, F, Tg, b, R);
+        } else {
+          merge_rows(top[buf], cc[buf], start, cnt, F);
+          const int ld = odd_ld(rows);
+          load_rows(P, lda, rows, bk, R, ld, F, true);
+          km = node_qr(R, ld, rows, bk, F, true, Tg, b, region_elems);
+          for (int k = warp; k < bk; k += kBW)
+            for (int p = lane; p < rows; p += 32)
+              if (k >= F.fz[p]) P[F.prow[p] + (size_t)k * lda] = R[p + (size_t)k * ld];
+        }
         if (tid == 0) {
           top[buf ^ 1][o] = top[buf][start];
           cc[buf ^ 1][o] = km;
