@@ -244,9 +244,11 @@ __global__ void __launch_bounds__(256, 1) trsv_flag_kernel(int n, int nrhs, cons
     }
     __syncthreads();
     if (abort_flag) return;
-    for (int idx = tid; idx < nbj * nrhs; idx += blockDim.x) {
-      const int k = idx % nbj, c = idx / nbj;
-      xj[k + c * kTb] = __ldcg(B + (c0 + k) + (size_t)c * ldb);
+    for (int idx = tid; idx < kTb * nrhs; idx += blockDim.x) {
+      const int k = idx % kTb, c = idx / kTb;
+      // zeros past a short block: the products there are with zeros of T, and
+      // what shared memory holds may not be finite
+      xj[k + c * kTb] = k < nbj ? __ldcg(B + (c0 + k) + (size_t)c * ldb) : 0.0;
     }
     __syncthreads();
     if (nrhs == 1) {  // one right-hand side: four independent partial sums

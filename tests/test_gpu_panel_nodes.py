@@ -181,3 +181,18 @@ def test_solve_sizes(ca, n, nrhs):
     ca.caqr_geqrs(Q, 64, ca.make_tree(128), qtree, Y)
     torch.cuda.synchronize()
     assert np.abs(to_host(Y) - X).max() <= 1e-11
+
+
+@pytest.mark.parametrize("n,nrhs", [(130, 16), (200, 3), (333, 16), (100, 9)])
+def test_solve_does_not_read_what_an_earlier_one_left(ca, n, nrhs):
+    """Rows past a short last block: a solve of NaN right-hand sides first, so
+    that whatever the same kernel left behind is not finite."""
+    A = inputs.gaussian(n, n, n) + 4.0 * np.sqrt(n) * np.eye(n)
+    X = inputs.gaussian(n, nrhs, 7)
+    F, Y, bad = to_dev(A), to_dev(A @ X), to_dev(np.full((n, nrhs), np.nan))
+    ipiv, _ = ca.calu_factor(F, 64, ca.make_tree(128))
+    for _ in range(40):
+        ca.calu_getrs(F, ipiv, bad.clone())
+    ca.calu_getrs(F, ipiv, Y)
+    torch.cuda.synchronize()
+    assert np.abs(to_host(Y) - X).max() <= 1e-11
