@@ -58,6 +58,15 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
                : "memory");
 }
 
+// One lane of the (converged) warp.  The compiler knows that what runs under it
+// is warp-uniform and keeps the operands of copies and MMAs in uniform
+// registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}\n" : "=r"(p));
+  return p != 0;
+}
+
 // Waits for the phase with parity `parity`; false after ~`limit` SM cycles.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, long long limit) {
   const uint32_t addr = smem_u32(bar);
@@ -119,30 +128,33 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
                : "memory");
 }
 
-// 32 TMEM lanes x 32 consecutive 32-bit columns; thread i of the warp gets
-// lane (lane base + i).
-__device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// Thread i of the warp gets TMEM lane (lane base + i).
+// 32 TMEM lanes x 4 consecutive 32-bit columns, without the wait
+__device__ __forceinline__ void tmem_ld_32x4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+// waits for the loads; every value passes through, so that no use of it moves up
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[8][4]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0][0]), "+r"(r[0][1]), "+r"(r[0][2]), "+r"(r[0][3]), "+r"(r[1][0]), "+r"(r[1][1]),
+                 "+r"(r[1][2]), "+r"(r[1][3]), "+r"(r[2][0]), "+r"(r[2][1]), "+r"(r[2][2]), "+r"(r[2][3]),
+                 "+r"(r[3][0]), "+r"(r[3][1]), "+r"(r[3][2]), "+r"(r[3][3]), "+r"(r[4][0]), "+r"(r[4][1]),
+                 "+r"(r[4][2]), "+r"(r[4][3]), "+r"(r[5][0]), "+r"(r[5][1]), "+r"(r[5][2]), "+r"(r[5][3])
+               :
+               : "memory");
+  asm volatile(""
+               : "+r"(r[6][0]), "+r"(r[6][1]), "+r"(r[6][2]), "+r"(r[6][3]), "+r"(r[7][0]), "+r"(r[7][1]),
+                 "+r"(r[7][2]), "+r"(r[7][3])
+               :
+               : "memory");
 }
 
-// 32 TMEM lanes x 8 consecutive 32-bit columns.
-__device__ __forceinline__ void tmem_ld_32x8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
 }
 
 // Shared-memory matrix descriptor of a K-major operand written by TMA with a
@@ -206,49 +218,60 @@ __device__ __forceinline__ double i64_scaled_to_double(long long v, int e2) {
   return __longlong_as_double((long long)(sign | ((unsigned long long)E << 52) | (m & ((1ull << 52) - 1))));
 }
 
-// v * 2^e2 as a double, rounded to nearest even: CUDA's correctly rounded
-// conversion of v, then the scale added to its exponent field (exact while
-// the result stays normal); zero and results outside the normal range take
-// the integer path above.
-__device__ __forceinline__ double scaled_rn(long long v, int e2) {
-  const long long bits = __double_as_longlong(__ll2double_rn(v));
-  const int E = (int)((bits >> 52) & 0x7ff) + e2;
-  if (v != 0 && E > 0 && E < 2047) return __longlong_as_double(bits + ((long long)e2 << 52));
-  return i64_scaled_to_double(v, e2);
-}
-
 // (hi 2^16 + lo) 2^e2 as a double, rounded once to nearest even, |hi| < 2^60
-// and |lo| < 2^40: the sum is brought to 64 normalized bits with a sticky last
-// one and rounded in integers, so the only FP64 instruction left is the
-// subtraction from C (7 digits: 119.6 -> 114.9 ms of updates at n = 10240;
-// with at most 5 digits one conversion of hi is cheaper).
-__device__ __forceinline__ double scaled_sum_rn(long long hi, long long lo, int e2) {
+// and |lo| < 2^40, without a branch and without the FP64 pipe (a conversion
+// costs that pipe as much as an add): the sum is brought to 64 normalized bits
+// with a sticky last one and rounded in integers.  slow: a sum of fewer than
+// 17 bits or a result outside the normal range -- scaled_sum_slow then.
+__device__ __forceinline__ double scaled_sum_rn(long long hi, long long lo, int e2, bool &slow) {
   hi += lo >> 16;                                  // floor: lo's low 16 bits stay non-negative
   unsigned long long w = (unsigned long long)(lo & 0xffff) << 48;  // bits below hi
   unsigned long long h = (unsigned long long)hi;
   const unsigned long long sign = h & (1ull << 63);
-  if (sign) {                                      // two's complement of the pair
-    w = 0ull - w;
-    h = ~h + (w == 0ull);
-  }
-  if (h == 0ull) {                                 // fewer than 17 bits (or none)
-    const double v = i64_scaled_to_double((long long)(w >> 48), e2);
-    return __longlong_as_double((long long)((unsigned long long)__double_as_longlong(v) | (v != 0.0 ? sign : 0ull)));
-  }
-  const int lz = __clzll((long long)h);            // >= 3
+  const unsigned long long m0 = (unsigned long long)(hi >> 63);
+  w = (w ^ m0) - m0;                               // two's complement of the pair when negative
+  h = (h ^ m0) + (m0 && w == 0ull ? 1ull : 0ull);
+  const int lz = __clzll((long long)(h | 1ull));   // >= 3
   unsigned long long n = (h << lz) | (w >> (64 - lz));
   n |= (w << lz) != 0ull;
   // n in [2^63, 2^64): value n 2^(e2 + 16 - lz), 53 bits kept
   const int E = 1023 + 63 + 16 - lz + e2;
-  if ((unsigned)(E - 1) >= 2045u) {                // outside the normal range: the slow path
-    const double v = i64_scaled_to_double((long long)(n >> 2) | (long long)((n & 3) != 0), e2 + 18 - lz);
-    return __longlong_as_double((long long)((unsigned long long)__double_as_longlong(v) | sign));
-  }
+  const bool zero = (h | w) == 0ull;
+  slow = !zero && (h == 0ull || (unsigned)(E - 1) >= 2045u);
   unsigned long long m = n >> 11;
   const unsigned rem = (unsigned)n & 0x7ffu;
-  m += (rem > 0x400u || (rem == 0x400u && (m & 1ull))) ? 1ull : 0ull;
+  m += (rem + (unsigned)(m & 1ull) > 0x400u) ? 1ull : 0ull;
   // a carry out of the 53 bits lands in the exponent
-  return __longlong_as_double((long long)(sign | (((unsigned long long)(E - 1) << 52) + m)));
+  return zero ? 0.0 : __longlong_as_double((long long)(sign | (((unsigned long long)(unsigned)(E - 1) << 52) + m)));
+}
+
+// hi 2^e2 by CUDA's correctly rounded conversion and an exponent add: cheaper
+// where there are no low digits (4 digits, n = 4096: 149 against 151 us).
+__device__ __forceinline__ double scaled_rn(long long hi, int e2, bool &slow) {
+  const long long bits = __double_as_longlong(__ll2double_rn(hi));
+  const int E = (int)((bits >> 52) & 0x7ff) + e2;
+  slow = hi != 0 && (unsigned)(E - 1) >= 2046u;
+  return hi == 0 ? 0.0 : __longlong_as_double(bits + ((long long)e2 << 52));
+}
+
+__device__ __noinline__ double scaled_sum_slow(long long hi, long long lo, int e2) {
+  hi += lo >> 16;
+  unsigned long long w = (unsigned long long)(lo & 0xffff) << 48, h = (unsigned long long)hi;
+  const bool neg = hi < 0;
+  if (neg) {
+    w = 0ull - w;
+    h = ~h + (w == 0ull);
+  }
+  double v;
+  if (h == 0ull) {
+    v = i64_scaled_to_double((long long)(w >> 48), e2);
+  } else {
+    const int lz = __clzll((long long)h);
+    unsigned long long n = (h << lz) | (w >> (64 - lz));
+    n |= (w << lz) != 0ull;
+    v = i64_scaled_to_double((long long)(n >> 2) | (long long)((n & 3) != 0), e2 + 18 - lz);
+  }
+  return neg ? -v : v;
 }
 
 // Digits of x for the split: F = round(|x| 2^(8S - e)) (|x| < 2^e), as a
@@ -352,7 +375,7 @@ __global__ void __launch_bounds__(256, 2)
   uint64_t *done = empty + 2;                                            // [1]
   uint32_t *tslot = (uint32_t *)(done + 1);
   volatile int *abort_flag = (volatile int *)(tslot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // uniform
   const int m0 = blockIdx.x * kTcBM, n0 = blockIdx.y * a.bn;
   const int item = blockIdx.z;
   const bool last = item == a.nbatch - 1;
@@ -379,7 +402,7 @@ __global__ void __launch_bounds__(256, 2)
   const uint32_t tmem = *tslot;
   int issued0 = 0, issued1 = 0;  // loads issued into stage 0 / 1
 
-  if (threadIdx.x == 0) {
+  if (warp == 0 && elect_one()) {
     // ---- producer: TMA loads of the digit tiles, one K block per stage ----
     for (int kb = 0; kb < a.kblocks; ++kb) {
       const int st = kb % a.nstages, round = kb / a.nstages;
@@ -401,10 +424,16 @@ __global__ void __launch_bounds__(256, 2)
       else
         ++issued1;
     }
-  } else if (threadIdx.x == 32) {
+  } else if (warp == 1 && elect_one()) {
     // ---- MMA issuer: digit products d_k d'_l with k + l <= S + 1 ----------
+    // The descriptors of a stage's slices differ by a constant, and whether a
+    // product starts its accumulator follows from the loop's indexes: a few
+    // instructions per MMA.  (Rebuilding both descriptors for every product
+    // took 229 clocks per MMA, six times the MMA itself.)
     const uint32_t idesc = idesc_bf16_f32(kTcBM, a.bn);
-    uint32_t started = 0;  // bit acc: accumulator acc already holds a product
+    const uint32_t stepA = (uint32_t)boxA >> 4, stepB = (uint32_t)boxB >> 4;
+    const int S = a.S, kst = a.bk / 16;
+    const int khalf0 = (64 + a.bk - 1) / a.bk;  // first K block of the second 64-wide half
     for (int kb = 0; kb < a.kblocks; ++kb) {
       const int st = kb % a.nstages;
       if (!mbar_wait(&full[st], (kb / a.nstages) & 1, kWaitLimit)) {
@@ -413,23 +442,32 @@ __global__ void __launch_bounds__(256, 2)
         break;
       }
       tc_fence_after();
-      uint8_t *sa = base + (size_t)st * stage_bytes;
-      uint8_t *sb = sa + (size_t)a.S * boxA;
-      const int khalf = (kb * a.bk >= 64) ? 1 : 0;  // which 64-wide half of K
-      for (int ka = 0; ka < a.S; ++ka)
-        for (int kq = 0; ka + kq < a.S; ++kq) {
-          // accumulator: the digit diagonal ka + kq; with 7 digits the last
-          // diagonal (7 products) is split by K block to stay below 2^24
+      const uint8_t *sa = base + (size_t)st * stage_bytes;
+      const uint64_t ad0 = sw_desc(smem_u32(sa), a.swz);
+      const uint64_t bd0 = sw_desc(smem_u32(sa + (size_t)S * boxA), a.swz);
+      // product d_ka d'_kq goes to the accumulator of its diagonal ka + kq
+      // (fused mode: 0); with 7 digits over two halves of K the last diagonal
+      // (7 products) has one accumulator per half, to stay below 2^24
+      const bool second = a.nacc == 8 && kb >= khalf0;
+      uint64_t ad = ad0;
+      for (int ka = 0; ka < S; ++ka) {
+        uint64_t bd = bd0;
+        for (int kq = 0; ka + kq < S; ++kq) {
           int acc = a.exact ? ka + kq : 0;
-          if (a.nacc == 8 && acc == 6) acc = 6 + khalf;
-          const uint32_t d = tmem + (uint32_t)(acc * a.bn);
-          const uint64_t ad = sw_desc(smem_u32(sa + (size_t)ka * boxA), a.swz);
-          const uint64_t bd = sw_desc(smem_u32(sb + (size_t)kq * boxB), a.swz);
-          for (int ks = 0; ks < a.bk / 16; ++ks) {  // +32 bytes of K per step
-            tc_mma(d, ad + 2 * ks, bd + 2 * ks, idesc, (started >> acc) & 1u);
-            started |= 1u << acc;
+          bool fresh = kb == 0 && ka == 0 && (a.exact || kq == 0);  // the accumulator holds nothing yet
+          if (second && acc == 6) {
+            acc = 7;
+            fresh = kb == khalf0 && ka == 0;
           }
+          const uint32_t d = tmem + (uint32_t)(acc * a.bn);
+          for (int ks = 0; ks < kst; ++ks) {  // +32 bytes of K per step
+            tc_mma(d, ad + 2 * ks, bd + 2 * ks, idesc, fresh ? 0u : 1u);
+            fresh = false;
+          }
+          bd += stepB;
         }
+        ad += stepA;
+      }
       tc_commit(&empty[st]);  // the stage may be refilled once these MMAs are done
     }
     tc_commit(done);
@@ -453,69 +491,84 @@ __global__ void __launch_bounds__(256, 2)
     // integers below 2^24; combine them in integer arithmetic,
     //   T_hi = sum_{D <= 4} acc_D 2^(8 (4 - D)),  T_lo = sum_{D > 4} acc_D 2^(8 (6 - D)),
     // and round their sum to a double once.
-    const int dmax = a.exact ? a.S - 1 : 0;
-    constexpr int kEp = 8;  // columns per epilogue step
-    for (int c0 = half * kEp; c0 < a.bn; c0 += 2 * kEp) {
-      long long thi[kEp], tlo[kEp];
+    // Four columns per step; the next step's C and exponents are on their way
+    // while this step's accumulators, all read at once, are combined.
+    constexpr int kEp = 4;
+    double cn[kEp];
+    int en[kEp];
+    auto fetch = [&](int c0) {
 #pragma unroll
-      for (int j = 0; j < kEp; ++j) thi[j] = tlo[j] = 0;
-      float vf[kEp];
-      // unrolled over the at most 8 accumulators: constant shifts
+      for (int j = 0; j < kEp; ++j) {
+        const int col = n0 + c0 + j;
+        const bool ok_c = rin && c0 < a.bn && col < nvv;
+        cn[j] = ok_c ? __ldcg(Cb + row + (size_t)col * a.ldc) : 0.0;
+        en[j] = ok_c ? __ldg(ebi + col) : 0;
+      }
+    };
+    fetch(half * kEp);
+    for (int c0 = half * kEp; c0 < a.bn; c0 += 2 * kEp) {
+      uint32_t r[8][kEp];
 #pragma unroll
       for (int d = 0; d < 8; ++d) {
-        if (d >= nacc) break;
-        uint32_t r[kEp];
-        tmem_ld_32x8(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(d * a.bn + c0), r);
-        if (!a.exact) {
-#pragma unroll
-          for (int j = 0; j < kEp; ++j) vf[j] = __uint_as_float(r[j]);
-          continue;
-        }
-        const int D = d < 7 ? d : 6;  // accumulator 7 is the second half of diagonal 6
-#pragma unroll
-        for (int j = 0; j < kEp; ++j) {
-          const long long q = (long long)__float2int_rn(__uint_as_float(r[j]));
-          if (D <= 4)
-            thi[j] += q << (8 * (4 - D));
-          else
-            tlo[j] += q << (8 * (6 - D));
-        }
+        r[d][0] = r[d][1] = r[d][2] = r[d][3] = 0u;
+        if (d < nacc) tmem_ld_32x4(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(d * a.bn + c0), r[d]);
       }
-      if (!rin) continue;
-      // all loads of C in flight before any store
       double cv[kEp];
       int ec[kEp];
 #pragma unroll
       for (int j = 0; j < kEp; ++j) {
-        const int col = n0 + c0 + j;
-        const bool ok_c = col < nvv;
-        cv[j] = ok_c ? __ldcg(Cb + row + (size_t)col * a.ldc) : 0.0;
-        ec[j] = ok_c ? __ldg(ebi + col) : 0;
+        cv[j] = cn[j];
+        ec[j] = en[j];
+      }
+      fetch(c0 + 2 * kEp);
+      tmem_ld_wait(r);
+      // straight-line for all columns of the step (a branch per element would
+      // run their long dependent chains one after the other)
+      unsigned slow = 0;
+      long long hi[kEp], lo[kEp];
+#pragma unroll
+      for (int j = 0; j < kEp; ++j) {
+        const int sc = er + ec[j] - 16;  // C -= sign 2^sc value
+        hi[j] = lo[j] = 0;
+        if (a.exact) {
+          // sum_D acc_D 2^(-8 D) = T_hi 2^(-32) + T_lo 2^(-48)
+#pragma unroll
+          for (int d = 0; d < 8; ++d) {
+            const int q = a.sign * __float2int_rn(__uint_as_float(r[d][j]));  // 0 beyond the accumulators
+            const int D = d < 7 ? d : 6;  // accumulator 7 is the second half of diagonal 6
+            if (D <= 4)
+              hi[j] = D == 0 ? (long long)q << 32 : mad_wide(q, 1 << (8 * (4 - D)), hi[j]);
+            else
+              lo[j] = mad_wide(q, 1 << (8 * (6 - D)), lo[j]);
+          }
+          bool sl;
+          cv[j] -= nacc > 5 ? scaled_sum_rn(hi[j], lo[j], sc - 48, sl) : scaled_rn(hi[j], sc - 32, sl);
+          slow |= (sl || (a.full && sc > kExOdd / 2)) ? 1u << j : 0u;
+        } else {
+          cv[j] = fma((double)(-a.sign * __uint_as_float(r[0][j])), pow2i(sc), cv[j]);
+        }
+      }
+      if (slow) {
+#pragma unroll
+        for (int j = 0; j < kEp; ++j) {
+          const int col = n0 + c0 + j;
+          if (!((slow >> j) & 1u) || !rin || col >= nvv) continue;
+          const int sc = er + ec[j] - 16;
+          const double c = __ldcg(Cb + row + (size_t)col * a.ldc);
+          cv[j] = (a.full && sc > kExOdd / 2) ? odd_element(a, item, row, col, c)
+                                              : c - scaled_sum_slow(hi[j], lo[j], sc - 48);
+        }
       }
 #pragma unroll
       for (int j = 0; j < kEp; ++j) {
         const int col = n0 + c0 + j;
-        if (col >= nvv) continue;
-        const int sc = er + ec[j] - 16;  // C -= sign 2^sc value
-        double c = cv[j];
-        if (a.full && sc > kExOdd / 2) {
-          c = odd_element(a, item, row, col, c);
-        } else if (a.exact) {
-          // value = T_hi 2^(8 (4 - dmax)) ... written relative to diagonal dmax:
-          // sum_D acc_D 2^(-8 D) = T_hi 2^(-32) + T_lo 2^(-48)
-          if (dmax > 4)
-            c -= scaled_sum_rn(a.sign > 0 ? thi[j] : -thi[j], a.sign > 0 ? tlo[j] : -tlo[j], sc - 48);
-          else
-            c -= scaled_rn(a.sign > 0 ? thi[j] : -thi[j], sc - 32);
-        } else {
-          c = fma((double)(-a.sign * vf[j]), pow2i(sc), c);
-        }
-        Cb[row + (size_t)col * a.ldc] = c;
+        if (rin && col < nvv) Cb[row + (size_t)col * a.ldc] = cv[j];
       }
     }
   }
   // every copy this CTA issued has landed before shared memory goes away
-  if (threadIdx.x == 0) {
+  // (the counts are the producer's)
+  if (issued0 + issued1 > 0) {
     if (issued0 > 0) mbar_wait(&full[0], (issued0 - 1) & 1, kWaitLimit);
     if (issued1 > 0) mbar_wait(&full[1], (issued1 - 1) & 1, kWaitLimit);
   }
@@ -673,7 +726,9 @@ struct TcCfg {
 // Tile width, K block and stages.  First choice: two CTAs of 8 warps per
 // SM (each with at most 256 tensor-memory columns and half the shared
 // memory), so that one CTA's epilogue -- the FP64 read-modify-write of its C
-// tile -- overlaps the other's loads and MMAs; tiles at least 64 wide.
+// tile -- overlaps the other's loads and MMAs; tiles at least 32 wide (5
+// digits, n = 4096: 231 us with two CTAs of 32-wide tiles, 268 with one of 64;
+// 7 digits 342 and 346).
 // Otherwise one CTA per SM: the widest tile whose accumulators fit in the
 // 512 columns.  Then the deepest K-block pipeline that fits in shared memory
 // (two stages overlap the loads of one K block with the MMAs of the
@@ -682,7 +737,7 @@ static bool tc_config(int S, int exact, int kpad, TcCfg &c) {
   const int nacc = tc_nacc(S, exact, kpad);
   {
     int bn2 = 128;
-    while (bn2 > 64 && nacc * bn2 > 256) bn2 /= 2;
+    while (bn2 > 32 && nacc * bn2 > 256) bn2 /= 2;
     if (nacc * bn2 <= 256) {
       const int opts2[3][2] = {{64, 2}, {32, 2}, {32, 1}};
       for (auto &o : opts2) {
