@@ -29,7 +29,7 @@
 // received every row j; the sender of row j passed the CTA barrier of step
 // j - 1, so all its warps are done with the rows j - 2 that the buffer held.
 // Measured (single node, before: shared-memory cluster kernel): 1024 x 128
-// 1310 -> 460 us, 512 x 128 520 -> 309 us, 128 x 64 200 -> 104 us, 96 x 96
+// 1310 -> 344 us, 512 x 128 520 -> 291 us, 128 x 64 200 -> 104 us, 96 x 96
 // 362 -> 180 us; leaf and merge rounds of 1048576 x 64 12.9 -> 8.6 ms.
 // The columns run in blocks of 4 TPR: register indices are constants inside a
 // block, and after a block the registers move down by 4, so the code stays
@@ -56,7 +56,7 @@ struct alignas(16) Key {
   int pad;
 };
 
-constexpr int kMaxG = 8;
+constexpr int kMaxG = 16;
 constexpr int kMaxWarps = 16;
 
 constexpr long long kLuWait = 4000000000ll;  // about 2 s of SM clock
@@ -453,6 +453,13 @@ __global__ void __launch_bounds__(lu_reg_rows<TPR, CPT>() * TPR, CPT == 16 && TP
 
 template <int TPR, int CPT, bool CL>
 cudaError_t launch_reg1(const TsluNodeArgs &a, int nodes, int G, cudaStream_t st) {
+  if (G > 8) {
+    static std::atomic<unsigned long long> big{0};
+    cudaError_t e = once_per_device(big, [] {
+      return cudaFuncSetAttribute(tslu_reg_kernel<TPR, CPT, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    });
+    if (e != cudaSuccess) return e;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nodes * G);
   cfg.blockDim = dim3((a.rloc * TPR + 31) / 32 * 32);
@@ -488,14 +495,16 @@ cudaError_t launch_reg(const TsluNodeArgs &a, int nodes, int G, cudaStream_t st)
 // smallest cluster that holds the rows, doubled while the round's CTAs still
 // find an SM each and a CTA keeps at least kMinRows rows (128 x 64: 125 us on
 // one CTA, 121 on 2, 104 on 4, 109 on 8; 256 x 64: 201, 150, 123, 109).
+// Sixteen CTAs (beyond the portable cluster size, so never needed to hold the
+// rows) for at most six nodes: 1024 x 128 471 -> 344 us, 512 x 128 317 -> 291.
 int tslu_reg_cluster(int R, int bk, int nodes, int *rloc) {
   if (bk < 1 || bk > 128 || R < 1) return 0;
   const int rmax = bk <= 64 ? 256 : 128;
   constexpr int kMinRows = 24;
   int G = 1;
-  while (G < kMaxG && (R + G - 1) / G > rmax) G *= 2;
+  while (G < 8 && (R + G - 1) / G > rmax) G *= 2;
   if ((R + G - 1) / G > rmax) return 0;
-  while (G < kMaxG && nodes * G * 2 <= 152 && (R + 2 * G - 1) / (2 * G) >= kMinRows) G *= 2;
+  while (G < kMaxG && (G < 8 || nodes * 16 <= 96) && nodes * G * 2 <= 152 && (R + 2 * G - 1) / (2 * G) >= kMinRows) G *= 2;
   *rloc = (R + G - 1) / G;
   return G;
 }
