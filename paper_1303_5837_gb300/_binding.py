@@ -28,6 +28,7 @@ CA_ERR_BATCH_ITEM = -1005
 CA_STATUS_NONFINITE = 1
 CA_STATUS_SOLVE_TIMEOUT = 16
 CA_STATUS_REFACTORED = 32
+CA_STATUS_PANEL_TIMEOUT = 64
 CA_REFINE_CLASSIC = 0
 CA_REFINE_GMRES = 1
 CA_REFINE_AUTO = 2

@@ -257,7 +257,7 @@ int caqr_run(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, dou
     cudaStream_t ps = la ? la->helper : stream;
     if (la && cudaStreamWaitEvent(ps, la->ev_next, 0) != cudaSuccess) return CA_ERR_LAUNCH;
     // 1. TSQR: leaves, then the R-elimination tree
-    if (tsqr_panel(mk, bk, b, P, lda, L, plan, Tp, ws, dev_info, ps) != cudaSuccess) return CA_ERR_LAUNCH;
+    if (tsqr_panel(mk, bk, b, P, lda, L, plan, Tp, ws, dev_info, ps, tcws != nullptr) != cudaSuccess) return CA_ERR_LAUNCH;
     if (la && (cudaEventRecord(la->ev_panel, ps) != cudaSuccess ||
                cudaStreamWaitEvent(stream, la->ev_panel, 0) != cudaSuccess))
       return CA_ERR_LAUNCH;

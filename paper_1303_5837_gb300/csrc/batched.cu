@@ -995,7 +995,7 @@ __device__ NodeRows<true> merge_rows_reg(const int *top, const int *c, int start
                                          Fixed<T> &F) {
   NodeRows<true> nr;
   nr.R = rows;
-  nr.reord = nr.beg = nr.c0 = nr.nk = nr.h = 0;
+  nr.reord = nr.beg = nr.c0 = nr.nk = nr.h = nr.fixed = 0;
   const int c0 = c[start], h = c[start + 1];
   bool same = true;
   for (int ch = 2; ch < cnt; ++ch) same &= c[start + ch] == h;

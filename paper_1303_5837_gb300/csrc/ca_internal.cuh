@@ -264,6 +264,7 @@ struct TsqrNodeArgs {
   int nleaves;
   int rloc, ld;   // tile rows per CTA, tile leading dimension (odd)
   int *dev_info;
+  int fixed;      // keep the order of sums and the library's square root (panel_qr_fixed.cu)
 };
 // Register-resident TSQR nodes (panel_qr_reg.cu) for nodes of at most 256
 // rows and 64 columns held by one CTA; *done = false when the shape is not
@@ -272,11 +273,13 @@ bool tsqr_reg_fits(int rows, int bk);
 // Whether a round of `nodes` nodes runs in the cluster form of the
 // register-resident node (up to 128 columns and 1024 rows).
 bool tsqr_creg_fits(int rows, int bk, int nodes);
+int tsqr_fixed_cluster(int rows, int bk);  // CTAs per node of panel_qr_fixed.cu, 0 when not covered
+cudaError_t launch_tsqr_fixed(const TsqrNodeArgs &a, int nodes, int rows, cudaStream_t st);
 cudaError_t launch_tsqr_creg(const TsqrNodeArgs &a, int nodes, int rows, cudaStream_t st);
 cudaError_t launch_tsqr_reg(const TsqrNodeArgs &a, int nodes, int rows, cudaStream_t st, bool *done);
 cudaError_t tsqr_panel(int mk, int bk, int b, double *P, int lda, int leaf_rows,
                        const Plan &plan, double *Tp, const QrPanelWs &ws, int *dev_info,
-                       cudaStream_t st);
+                       cudaStream_t st, bool fixed = false);
 cudaError_t tree_apply_qt(int mk, int bk, int b, const double *P, int lda, int leaf_rows,
                           const Plan &plan, const double *Tp, double *C, int ldc, int ncols,
                           const QrPanelWs &ws, cudaStream_t st);

@@ -931,6 +931,7 @@ static cudaError_t launch_tsqr_node(const TsqrNodeArgs &args, int nodes, int G, 
     e = launch_tsqr_reg(args, nodes, (int)r, st, &done);
     return (e == cudaSuccess && !done) ? cudaErrorInvalidValue : e;
   }
+  if (G < 0 && args.fixed) return launch_tsqr_fixed(args, nodes, (int)r, st);
   if (G < 0) return launch_tsqr_creg(args, nodes, (int)r, st);  // registers of a cluster
   cfg.gridDim = dim3(nodes * G);
   cfg.blockDim = dim3(kQrThreads);
@@ -947,7 +948,7 @@ static cudaError_t launch_tsqr_node(const TsqrNodeArgs &args, int nodes, int G, 
 }
 
 cudaError_t tsqr_panel(int mk, int bk, int b, double *P, int lda, int leaf_rows, const Plan &plan,
-                       double *Tp, const QrPanelWs &ws, int *dev_info, cudaStream_t st) {
+                       double *Tp, const QrPanelWs &ws, int *dev_info, cudaStream_t st, bool fixed) {
   TsqrNodeArgs a = {};
   a.P = P;
   a.lda = lda;
@@ -958,12 +959,15 @@ cudaError_t tsqr_panel(int mk, int bk, int b, double *P, int lda, int leaf_rows,
   a.Tp = Tp;
   a.nleaves = plan.nleaves;
   a.dev_info = dev_info;
+  a.fixed = fixed ? 1 : 0;
   int R = leaf_rows < mk ? leaf_rows : mk;
   int rloc = 0, ld = 0;
-  // G = 0: the register-resident node kernel; -1: its cluster form; else
+  // G = 0: the register-resident node kernel; -1: its cluster form (fixed: the
+  // one with the fixed order of sums); else
   // the shared-memory node kernel on a cluster of G CTAs
   auto pick = [&](int rows, int nodes) {
-    if (tsqr_creg_fits(rows, bk, nodes)) return -1;
+    if (fixed && tsqr_fixed_cluster(rows, bk) >= 2) return -1;
+    if (!fixed && tsqr_creg_fits(rows, bk, nodes)) return -1;
     if (tsqr_reg_fits(rows, bk)) return 0;
     const int g = pick_qr_cluster(rows, bk, nodes, &rloc, &ld);
     return g > 0 ? g : -2;

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(kRegThreads, reg_min_blocks<TC, TS>()) tsqr_re
   nr.reord = 0;
   nr.beg = 0;
   nr.c0 = nr.nk = nr.h = 0;
+  nr.fixed = a.fixed;
   if (!a.is_leaf) {
     const int c0 = a.c_in[start], h = a.c_in[start + 1];
     bool same = true;

@@ -20,7 +20,33 @@ struct RegSmem {
 // below it: beta = -sign(alpha) ||(alpha, x)||, tau = (beta - alpha) / beta,
 // s = 1 / (alpha - beta).  Three dependent FP64 instructions and integer work
 // (about 470 clocks; a square root and two divisions take 2000).
-__device__ __forceinline__ void reflector(double alpha, double ss, double &beta, double &tau, double &s) {
+static __device__ __noinline__ void reflector_lib(double alpha, double ss, double &beta, double &tau, double &s) {
+  const double nrm = sqrt(fma(alpha, alpha, ss));
+  beta = (alpha >= 0.0) ? -nrm : nrm;
+  tau = (beta - alpha) / beta;
+  s = 1.0 / (alpha - beta);
+}
+// The same three values bit for bit: square root and quotient by Markstein's
+// final step (the exact residual of an approximation times its reciprocal,
+// added to it), correctly rounded from approximations this close; the
+// reciprocals correctly rounded in integers.
+__device__ __forceinline__ void reflector_fixed(double alpha, double ss, double &beta, double &tau, double &s) {
+  const double v = fma(alpha, alpha, ss);
+  if (!int_range(v)) return reflector_lib(alpha, ss, beta, tau, s);
+  const double y = rsqrt_near(v), q = v * y;
+  const double nrm = fma(0.5 * y, fma(-q, q, v), q);
+  const double be = (alpha >= 0.0) ? -nrm : nrm;
+  const double num = be - alpha, rb = recip_exact_or_zero(be), rd = recip_exact_or_zero(-num);
+  if (__double_as_longlong(rb) == 0 || __double_as_longlong(rd) == 0) return reflector_lib(alpha, ss, beta, tau, s);
+  const double z = num * rb;
+  beta = be;
+  tau = fma(fma(-z, be, num), rb, z);
+  s = rd;
+}
+// fixed: correctly rounded (panel_qr_fixed.cu)
+__device__ __forceinline__ void reflector(double alpha, double ss, double &beta, double &tau, double &s,
+                                          bool fixed = false) {
+  if (fixed) return reflector_fixed(alpha, ss, beta, tau, s);
   const double v = fma(alpha, alpha, ss), a = fabs(alpha);
   if (int_range(v)) {
     const double y = rsqrt_near(v);
@@ -31,14 +57,10 @@ __device__ __forceinline__ void reflector(double alpha, double ss, double &beta,
     beta = neg ? nrm : -nrm;
     s = neg ? -r : r;
   } else {
-    const double nrm = sqrt(v);
-    beta = (alpha >= 0.0) ? -nrm : nrm;
-    tau = (beta - alpha) / beta;
-    s = 1.0 / (alpha - beta);
+    reflector_lib(alpha, ss, beta, tau, s);
   }
 }
-
-__device__ __forceinline__ void reflector(float alpha, float ss, float &beta, float &tau, float &s) {
+__device__ __forceinline__ void reflector(float alpha, float ss, float &beta, float &tau, float &s, bool = false) {
   const float nrm = sqrtf(fmaf(alpha, alpha, ss));
   beta = (alpha >= 0.0f) ? -nrm : nrm;
   tau = (beta - alpha) / beta;
@@ -94,6 +116,7 @@ struct NodeRows {
   int reord;  // 1: merge rows in the order above
   int beg;    // first block that can hold such rows
   int c0, nk, h, R;
+  int fixed;  // correctly rounded reflectors (reflector_fixed)
   // leaves run every block (the zero rows of a short leaf cost nothing wrong)
   __device__ __forceinline__ int first() const { return MERGE ? beg : 0; }
   __device__ __forceinline__ int end(int j) const {
@@ -124,7 +147,7 @@ __device__ __forceinline__ void reflect(F (&A)[TS][TC], const NodeRows<MERGE> &n
   F t = F(0), sc = F(1);
   if (ss != F(0)) {
     F beta;
-    reflector(alpha, ss, beta, t, sc);
+    reflector(alpha, ss, beta, t, sc, nr.fixed != 0);
     if (rg == jr) A[U][U] = beta;
   }
 #pragma unroll
