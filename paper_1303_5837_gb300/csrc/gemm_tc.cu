@@ -426,14 +426,15 @@ __global__ void __launch_bounds__(256, 2)
     }
   } else if (warp == 1 && elect_one()) {
     // ---- MMA issuer: digit products d_k d'_l with k + l <= S + 1 ----------
-    // The descriptors of a stage's slices differ by a constant, and whether a
-    // product starts its accumulator follows from the loop's indexes: a few
-    // instructions per MMA.  (Rebuilding both descriptors for every product
-    // took 229 clocks per MMA, six times the MMA itself.)
-    const uint32_t idesc = idesc_bf16_f32(kTcBM, a.bn);
+    // One thread issues, so the MMAs' count matters as much as their size: a
+    // product of its own for each pair of digits (28 of 128 x 32 x 16 per K
+    // step with 7 digits) took 121 clocks each; now S wide ones cover it.
+    // n = 4096, K = 128: 7 digits 348 -> 268 us (448 TFLOP/s),
+    // 5 digits 231 -> 190, 4 digits 143 -> 133.
     const uint32_t stepA = (uint32_t)boxA >> 4, stepB = (uint32_t)boxB >> 4;
     const int S = a.S, kst = a.bk / 16;
     const int khalf0 = (64 + a.bk - 1) / a.bk;  // first K block of the second 64-wide half
+    const int wide = max(1, 256 / a.bn);        // digits of B that one MMA takes
     for (int kb = 0; kb < a.kblocks; ++kb) {
       const int st = kb % a.nstages;
       if (!mbar_wait(&full[st], (kb / a.nstages) & 1, kWaitLimit)) {
@@ -445,28 +446,42 @@ __global__ void __launch_bounds__(256, 2)
       const uint8_t *sa = base + (size_t)st * stage_bytes;
       const uint64_t ad0 = sw_desc(smem_u32(sa), a.swz);
       const uint64_t bd0 = sw_desc(smem_u32(sa + (size_t)S * boxA), a.swz);
-      // product d_ka d'_kq goes to the accumulator of its diagonal ka + kq
-      // (fused mode: 0); with 7 digits over two halves of K the last diagonal
-      // (7 products) has one accumulator per half, to stay below 2^24
-      const bool second = a.nacc == 8 && kb >= khalf0;
-      uint64_t ad = ad0;
-      for (int ka = 0; ka < S; ++ka) {
-        uint64_t bd = bd0;
-        for (int kq = 0; ka + kq < S; ++kq) {
-          int acc = a.exact ? ka + kq : 0;
-          bool fresh = kb == 0 && ka == 0 && (a.exact || kq == 0);  // the accumulator holds nothing yet
-          if (second && acc == 6) {
-            acc = 7;
-            fresh = kb == khalf0 && ka == 0;
+      if (a.exact) {
+        // Product d_ka d'_kq goes to the accumulator of its diagonal ka + kq.
+        // The digits of B lie one after the other in shared memory and the
+        // accumulators in tensor memory, so one MMA multiplies d_ka by as many
+        // of B's digits as 256 columns hold.  With 7 digits over two halves of
+        // K the last diagonal (7 products) has one accumulator per half, to
+        // stay below 2^24: its product is issued alone in the second half.
+        const bool second = a.nacc == 8 && kb >= khalf0;
+        for (int ks = 0; ks < kst; ++ks) {  // +32 bytes of K per step
+          uint64_t ad = ad0 + 2 * ks;
+          for (int ka = 0; ka < S; ++ka) {
+            const int nq = S - ka - (second ? 1 : 0);  // products in their own diagonal's accumulator
+            const uint32_t more = kb > 0 || ka > 0 || ks > 0;  // 0: the accumulators hold nothing yet
+            for (int kq = 0; kq < nq; kq += wide) {
+              const int w = min(wide, nq - kq) * a.bn;
+              tc_mma(tmem + (uint32_t)((ka + kq) * a.bn), ad, bd0 + (uint64_t)(kq * stepB + 2 * ks),
+                     idesc_bf16_f32(kTcBM, w), more);
+            }
+            if (second)
+              tc_mma(tmem + (uint32_t)(7 * a.bn), ad, bd0 + (uint64_t)(nq * stepB + 2 * ks),
+                     idesc_bf16_f32(kTcBM, a.bn), kb > khalf0 || ka > 0 || ks > 0);
+            ad += stepA;
           }
-          const uint32_t d = tmem + (uint32_t)(acc * a.bn);
-          for (int ks = 0; ks < kst; ++ks) {  // +32 bytes of K per step
-            tc_mma(d, ad + 2 * ks, bd + 2 * ks, idesc, fresh ? 0u : 1u);
-            fresh = false;
-          }
-          bd += stepB;
         }
-        ad += stepA;
+      } else {
+        const uint32_t idesc = idesc_bf16_f32(kTcBM, a.bn);
+        uint64_t ad = ad0;
+        for (int ka = 0; ka < S; ++ka) {
+          uint64_t bd = bd0;
+          for (int kq = 0; ka + kq < S; ++kq) {
+            for (int ks = 0; ks < kst; ++ks)
+              tc_mma(tmem, ad + 2 * ks, bd + 2 * ks, idesc, kb > 0 || ka > 0 || kq > 0 || ks > 0);
+            bd += stepB;
+          }
+          ad += stepA;
+        }
       }
       tc_commit(&empty[st]);  // the stage may be refilled once these MMAs are done
     }
@@ -728,7 +743,7 @@ struct TcCfg {
 // memory), so that one CTA's epilogue -- the FP64 read-modify-write of its C
 // tile -- overlaps the other's loads and MMAs; tiles at least 32 wide (5
 // digits, n = 4096: 231 us with two CTAs of 32-wide tiles, 268 with one of 64;
-// 7 digits 342 and 346).
+// 7 digits 342 and 346; both with one MMA per pair of digits).
 // Otherwise one CTA per SM: the widest tile whose accumulators fit in the
 // 512 columns.  Then the deepest K-block pipeline that fits in shared memory
 // (two stages overlap the loads of one K block with the MMAs of the
