@@ -111,6 +111,20 @@ def test_qr_node_shapes(ca, m, n, L, lv):
     qr_case(ca, inputs.gaussian(m, n, 13 * m + n), L, lv)
 
 
+@pytest.mark.parametrize("m,n,L,lv", [c for c in QR_NODES if c[1] > 1] + [(512, 70, 512, [(0, 0)])])
+def test_qr_node_shapes_of_the_digit_form(ca, m, n, L, lv):
+    """One panel of the digit factorization, which keeps its own order of sums."""
+    A = inputs.gaussian(m, n, 13 * m + n)
+    t_o = oracle.make_tree(L, lv)
+    QR_o, T_o = oracle.caqr(A, n, t_o)
+    Ad = to_dev(A)
+    qtree, info = ca.caqr_factor_mixed(Ad, n, ca.make_tree(L, lv))
+    torch.cuda.synchronize()
+    assert info.cpu().tolist() == [0, 0]
+    check(qr_err(to_host(Ad), QR_o), TOL, (m, n, L))
+    check(qtree_err(qtree.cpu().numpy(), T_o, QR_o, n, t_o, oracle.tree_counts), TOL, (m, n, L))
+
+
 @pytest.mark.parametrize("scale", [1e-200, 1e150, 1e-305])
 @pytest.mark.parametrize("m,n,L", [(200, 24, 100), (600, 100, 300)])
 def test_qr_node_reflectors_at_the_ends_of_the_range(ca, m, n, L, scale):
