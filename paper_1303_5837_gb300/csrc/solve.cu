@@ -251,11 +251,11 @@ __global__ void __launch_bounds__(256, 1) trsv_flag_kernel(int n, int nrhs, cons
       xj[k + c * kTb] = k < nbj ? __ldcg(B + (c0 + k) + (size_t)c * ldb) : 0.0;
     }
     __syncthreads();
-    if (nrhs == 1) {  // one right-hand side: four independent partial sums
-      double a4[4] = {0.0, 0.0, 0.0, 0.0};
+    if (nrhs == 1) {  // one right-hand side: two independent partial sums (four take as long)
+      double a2[2] = {0.0, 0.0};
 #pragma unroll
-      for (int k = 0; k < kKp; ++k) a4[k & 3] = fma(trow[k], xj[k0 + k], a4[k & 3]);
-      part[half * kTb * kCoopMaxRhs + r] = (a4[0] + a4[1]) + (a4[2] + a4[3]);
+      for (int k = 0; k < kKp; ++k) a2[k & 1] = fma(trow[k], xj[k0 + k], a2[k & 1]);
+      part[half * kTb * kCoopMaxRhs + r] = a2[0] + a2[1];
     } else {
       double acc[kCoopMaxRhs];
 #pragma unroll
