@@ -990,9 +990,8 @@ __device__ int merge_rows(const int *top, const int *c, int start, int cnt, Fixe
 
 // The same for a node in registers: the other children's rows in the order of
 // their index within the child where all have one height (NodeRows).
-template <class T>
 __device__ NodeRows<true> merge_rows_reg(const int *top, const int *c, int start, int cnt, int rows, int kmax,
-                                         Fixed<T> &F) {
+                                         Fixed<double> &F) {
   NodeRows<true> nr;
   nr.R = rows;
   nr.reord = nr.beg = nr.c0 = nr.nk = nr.h = nr.fixed = 0;
@@ -1020,17 +1019,25 @@ __device__ NodeRows<true> merge_rows_reg(const int *top, const int *c, int start
 // A QR node in registers (qr_node_reg.cuh): loads the rows F.prow[0..rows) of
 // the panel (zero left of F.fz in a merge), factors them, writes the rows and
 // T back.  nr: the order of the rows (a merge's may be reordered).  The
-// shared-memory tile it replaces (node_qr) takes four barriers and a serial
-// reflector per column and three shared-memory accesses per multiply-add.
-template <class T, int TC, int TS>
-__device__ __noinline__ int node_qr_reg(T *P, int lda, int rows, int bk, const NodeRows<true> &nr, bool use_fz,
-                                        Fixed<T> &F, T *Tg, int b, T *R) {
-  RegSmem<T, TC, TS> &sm = *reinterpret_cast<RegSmem<T, TC, TS> *>(R);
+// shared-memory tile (node_qr) takes four barriers and a serial reflector per
+// column and three shared-memory accesses per multiply-add: the FP64 batch of
+// 1024 items takes 144.8 ms with it, 142.1 with this one.
+// FP64 only: the sums run over x unscaled and in another order, which in FP32
+// moves single elements of T by a thousand units of rounding (the last
+// reflectors of a square item come from sub-columns of one or two rows).  And
+// only where a product of two elements can neither underflow nor overflow;
+// otherwise -1 is returned and nothing has been written (node_qr sums
+// x / (alpha - beta), whose elements are at most one).
+template <int TC, int TS>
+__device__ __noinline__ int node_qr_reg(double *P, int lda, int rows, int bk, const NodeRows<true> &nr, bool use_fz,
+                                        Fixed<double> &F, double *Tg, int b, double *R) {
+  using T = double;
+  RegSmem<TC, TS> &sm = *reinterpret_cast<RegSmem<TC, TS> *>(R);
   const int tid = threadIdx.x, lane = tid & 31;
   const int rg = lane & 15, cg = 2 * (tid >> 5) + (lane >> 4);
   const int kmax = min(rows, bk);
   T A[TS][TC];
-  bool bad = false;
+  bool bad = false, wide = false;
 #pragma unroll
   for (int s = 0; s < TS; ++s) {
     const int p = rg + 16 * s;
@@ -1041,11 +1048,14 @@ __device__ __noinline__ int node_qr_reg(T *P, int lda, int rows, int bk, const N
       T v = T(0);
       if (prow >= 0 && q < bk && q >= fz) v = P[prow + (size_t)q * lda];
       bad |= Num<T>::bad(v);
+      const unsigned long long av = absbits(v);
+      wide |= av != 0ull && (unsigned)(av >> 52) - 623u > 800u;  // outside 2^-400 .. 2^400
       A[s][t] = v;
     }
   }
+  if (__syncthreads_or(wide && !bad)) return -1;
   if (bad) atomicOr(&F.status, CA_STATUS_NONFINITE);
-  qr_node<T, TC, TS, true>(A, nr, sm, kmax);
+  qr_node<TC, TS, true>(A, nr, sm, kmax);
   for (int idx = tid; idx < b * b; idx += kBT) {
     const int i = idx % b, jj = idx / b;
     T v = T(0);
@@ -1068,11 +1078,10 @@ __device__ __noinline__ int node_qr_reg(T *P, int lda, int rows, int bk, const N
 // Nodes of up to 512 rows and 32 columns, or 256 rows and 64 columns.
 __device__ __forceinline__ bool qr_reg_fits(int rows, int bk) { return bk <= 32 ? rows <= 512 : bk <= 64 && rows <= 256; }
 
-template <class T>
-__device__ __forceinline__ int node_qr_regs(T *P, int lda, int rows, int bk, const NodeRows<true> &nr, bool use_fz,
-                                            Fixed<T> &F, T *Tg, int b, T *R) {
-  return bk > 32 ? node_qr_reg<T, 4, 16>(P, lda, rows, bk, nr, use_fz, F, Tg, b, R)
-                 : node_qr_reg<T, 2, 32>(P, lda, rows, bk, nr, use_fz, F, Tg, b, R);
+__device__ __forceinline__ int node_qr_regs(double *P, int lda, int rows, int bk, const NodeRows<true> &nr, bool use_fz,
+                                            Fixed<double> &F, double *Tg, int b, double *R) {
+  return bk > 32 ? node_qr_reg<4, 16>(P, lda, rows, bk, nr, use_fz, F, Tg, b, R)
+                 : node_qr_reg<2, 32>(P, lda, rows, bk, nr, use_fz, F, Tg, b, R);
 }
 
 // C <- Q_node^T C for the node rows F.prow[0..rows) (leaf: Y unit lower
@@ -1257,12 +1266,15 @@ __device__ void cta_caqr(const ca_batch_item_t &it, Fixed<T> &F, T *R, int regio
       const int r0 = j * L, rows = min(L, mk - r0), ld = odd_ld(rows);
       for (int p = tid; p < rows; p += kBT) F.prow[p] = r0 + p;
       __syncthreads();
-      int km;
-      if (qr_reg_fits(rows, bk)) {
-        NodeRows<true> nr = {};
-        nr.R = rows;  // every row block takes part
-        km = node_qr_regs(P, lda, rows, bk, nr, false, F, Tp + (size_t)j * b * b, b, R);
-      } else {
+      int km = -1;
+      if constexpr (sizeof(T) == 8) {
+        if (qr_reg_fits(rows, bk)) {
+          NodeRows<true> nr = {};
+          nr.R = rows;  // every row block takes part
+          km = node_qr_regs(P, lda, rows, bk, nr, false, F, Tp + (size_t)j * b * b, b, R);
+        }
+      }
+      if (km < 0) {
         load_rows(P, lda, rows, bk, R, ld, F, false);
         km = node_qr(R, ld, rows, bk, F, false, Tp + (size_t)j * b * b, b, region_elems);
         for (int k = warp; k < bk; k += kBW)
@@ -1289,15 +1301,18 @@ __device__ void cta_caqr(const ca_batch_item_t &it, Fixed<T> &F, T *R, int regio
           __syncthreads();
           continue;
         }
-        int rows = 0;
-        for (int ch = 0; ch < cnt; ++ch) rows += cc[buf][start + ch];
         T *Tg = Tp + (size_t)(nl + midx) * b * b;
-        int km;
-        if (qr_reg_fits(rows, bk)) {
-          const NodeRows<true> nr = merge_rows_reg(top[buf], cc[buf], start, cnt, rows, min(rows, bk), F);
-          km = node_qr_regs(P, lda, rows, bk, nr, true, F, Tg, b, R);
-        } else {
-          merge_rows(top[buf], cc[buf], start, cnt, F);
+        int km = -1;
+        if constexpr (sizeof(T) == 8) {
+          int rows = 0;
+          for (int ch = 0; ch < cnt; ++ch) rows += cc[buf][start + ch];
+          if (qr_reg_fits(rows, bk)) {
+            const NodeRows<true> nr = merge_rows_reg(top[buf], cc[buf], start, cnt, rows, min(rows, bk), F);
+            km = node_qr_regs(P, lda, rows, bk, nr, true, F, Tg, b, R);
+          }
+        }
+        if (km < 0) {
+          const int rows = merge_rows(top[buf], cc[buf], start, cnt, F);
           const int ld = odd_ld(rows);
           load_rows(P, lda, rows, bk, R, ld, F, true);
           km = node_qr(R, ld, rows, bk, F, true, Tg, b, region_elems);

@@ -41,7 +41,7 @@ constexpr int reg_min_blocks() {
 
 template <int TC, int TS, bool MERGE>
 __global__ void __launch_bounds__(kRegThreads, reg_min_blocks<TC, TS>()) tsqr_reg_kernel(TsqrNodeArgs a) {
-  __shared__ RegSmem<double, TC, TS> sm;
+  __shared__ RegSmem<TC, TS> sm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rg = lane & 15, cg = 2 * warp + (lane >> 4);
   const int node = blockIdx.x;
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kRegThreads, reg_min_blocks<TC, TS>()) tsqr_re
   if (bad && a.dev_info) atomicOr(a.dev_info + 1, CA_STATUS_NONFINITE);
 
   // ---- Householder QR, one barrier per column, and T -----------------------
-  qr_node<double, TC, TS, MERGE>(A, nr, sm, kmax);
+  qr_node<TC, TS, MERGE>(A, nr, sm, kmax);
   {
     const int b = a.b;
     double *Tg = a.Tp + (size_t)(a.is_leaf ? node : a.nleaves + midx) * b * b;

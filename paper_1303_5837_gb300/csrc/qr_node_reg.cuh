@@ -1,5 +1,5 @@
 // qr_node_reg.cuh -- Householder QR of one tree node in the registers of a CTA
-// of 256 threads, in FP64 or FP32 (panel_qr_reg.cu, batched.cu).
+// of 256 threads (panel_qr_reg.cu, batched.cu).
 #pragma once
 #include "ca_internal.cuh"
 #include "fp64_int.cuh"
@@ -8,12 +8,12 @@ namespace cagb {
 
 constexpr int kRegThreads = 256;
 
-template <class F, int TC, int TS>
+template <int TC, int TS>
 struct RegSmem {
-  F xs[2][16 * TS];                 // x of the published column, by column parity
-  F tau[16 * TC], scal[16 * TC];    // tau_q, s_q (1 when tau_q = 0)
-  F Z[16 * TC * (16 * TC - 1) / 2];  // v_i^T v_j, i < j, at j (j - 1) / 2 + i
-  F T[16 * TC * (16 * TC - 1) / 2];  // strict upper part of T, same packing
+  double xs[2][16 * TS];                 // x of the published column, by column parity
+  double tau[16 * TC], scal[16 * TC];    // tau_q, s_q (1 when tau_q = 0)
+  double Z[16 * TC * (16 * TC - 1) / 2];  // v_i^T v_j, i < j, at j (j - 1) / 2 + i
+  double T[16 * TC * (16 * TC - 1) / 2];  // strict upper part of T, same packing
 };
 
 // The reflector of a column with diagonal alpha and sum of squares ss != 0
@@ -60,13 +60,6 @@ __device__ __forceinline__ void reflector(double alpha, double ss, double &beta,
     reflector_lib(alpha, ss, beta, tau, s);
   }
 }
-__device__ __forceinline__ void reflector(float alpha, float ss, float &beta, float &tau, float &s, bool = false) {
-  const float nrm = sqrtf(fmaf(alpha, alpha, ss));
-  beta = (alpha >= 0.0f) ? -nrm : nrm;
-  tau = (beta - alpha) / beta;
-  s = 1.0f / (alpha - beta);
-}
-
 // Sum of e[t] over the 16 lanes of the half-warp by reduce-scatter: lane rg
 // gets the sum of value t = sum_index<TC>(rg).
 template <int TC>
@@ -79,10 +72,10 @@ __device__ __forceinline__ int sum_lane(int t) {  // a lane that holds the sum o
   constexpr int L = TC == 1 ? 0 : TC == 2 ? 1 : TC == 4 ? 2 : 3;
   return t << (4 - L);
 }
-template <int TC, class F>
-__device__ __forceinline__ F half_sum_scatter(const F (&e)[TC], int rg) {
+template <int TC>
+__device__ __forceinline__ double half_sum_scatter(const double (&e)[TC], int rg) {
   constexpr int L = TC == 1 ? 0 : TC == 2 ? 1 : TC == 4 ? 2 : 3;
-  F v[TC];
+  double v[TC];
 #pragma unroll
   for (int t = 0; t < TC; ++t) v[t] = e[t];
 #pragma unroll
@@ -92,8 +85,8 @@ __device__ __forceinline__ F half_sum_scatter(const F (&e)[TC], int rg) {
     const bool up = (rg & o) != 0;
 #pragma unroll
     for (int i = 0; i < h; ++i) {
-      const F keep = up ? v[i + h] : v[i];
-      const F send = up ? v[i] : v[i + h];
+      const double keep = up ? v[i + h] : v[i];
+      const double send = up ? v[i] : v[i + h];
       v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o, 16);
     }
   }
@@ -129,12 +122,12 @@ struct NodeRows {
 // Reflector of column jc = 16 U + jr, by the half-warp that holds it (cg =
 // jr): beta = -sign(alpha) ||(alpha, x)||, tau = (beta - alpha) / beta,
 // s = 1 / (alpha - beta); R(jc, jc) = beta; x published to xs.
-template <class F, int TC, int TS, int U, bool MERGE>
-__device__ __forceinline__ void reflect(F (&A)[TS][TC], const NodeRows<MERGE> &nr, int rg, int jr, int jc,
-                                        F *xs, F *tau, F *scal) {
+template <int TC, int TS, int U, bool MERGE>
+__device__ __forceinline__ void reflect(double (&A)[TS][TC], const NodeRows<MERGE> &nr, int rg, int jr, int jc,
+                                        double *xs, double *tau, double *scal) {
   const unsigned hm = 0xffffu << (threadIdx.x & 16);
   const int se = nr.end(jc);
-  F ss = F(0);
+  double ss = 0.0;
 #pragma unroll
   for (int s = U; s < TS; ++s) {
     if (s >= se) break;
@@ -143,10 +136,10 @@ __device__ __forceinline__ void reflect(F (&A)[TS][TC], const NodeRows<MERGE> &n
   }
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(hm, ss, o, 16);
-  const F alpha = __shfl_sync(hm, A[U][U], jr, 16);
-  F t = F(0), sc = F(1);
-  if (ss != F(0)) {
-    F beta;
+  const double alpha = __shfl_sync(hm, A[U][U], jr, 16);
+  double t = 0.0, sc = 1.0;
+  if (ss != 0.0) {
+    double beta;
     reflector(alpha, ss, beta, t, sc, nr.fixed != 0);
     if (rg == jr) A[U][U] = beta;
   }
@@ -154,7 +147,7 @@ __device__ __forceinline__ void reflect(F (&A)[TS][TC], const NodeRows<MERGE> &n
   for (int s = U; s < TS; ++s) {
     if (s >= se) break;
     if (s < nr.first()) continue;
-    xs[16 * s + rg] = (s > U || rg > jr) ? A[s][U] : F(0);
+    xs[16 * s + rg] = (s > U || rg > jr) ? A[s][U] : 0.0;
   }
   if (rg == 0) {
     tau[jc] = t;
@@ -164,9 +157,9 @@ __device__ __forceinline__ void reflect(F (&A)[TS][TC], const NodeRows<MERGE> &n
 
 // A(:, q) -= v_j w_q for the thread's column t (q = cg + 16 t > j): row j
 // takes w_q itself, rows below it x_i s_j w_q (x is zero at rows <= j).
-template <class F, int TC, int TS, int U>
-__device__ __forceinline__ void update_col(F (&A)[TS][TC], const F (&x)[TS], int sb, int se, int t, F wt, F sw,
-                                           bool row_j) {
+template <int TC, int TS, int U>
+__device__ __forceinline__ void update_col(double (&A)[TS][TC], const double (&x)[TS], int sb, int se, int t,
+                                           double wt, double sw, bool row_j) {
 #pragma unroll
   for (int s = U; s < TS; ++s) {
     if (s >= se) break;
@@ -177,33 +170,33 @@ __device__ __forceinline__ void update_col(F (&A)[TS][TC], const F (&x)[TS], int
 }
 
 // Columns j = 16 U .. 16 U + 15 (those below kmax); row blocks [sb, se).
-template <class F, int TC, int TS, int U, bool MERGE>
-__device__ __forceinline__ void qr_block(F (&A)[TS][TC], const NodeRows<MERGE> &nr, RegSmem<F, TC, TS> &sm,
+template <int TC, int TS, int U, bool MERGE>
+__device__ __forceinline__ void qr_block(double (&A)[TS][TC], const NodeRows<MERGE> &nr, RegSmem<TC, TS> &sm,
                                          int rg, int cg, int kmax) {
   for (int jr = 0; jr < 16; ++jr) {
     const int j = 16 * U + jr;
     if (j >= kmax) return;
     __syncthreads();  // column j's x, tau_j and s_j are published
-    const F tj = sm.tau[j], sj = sm.scal[j];
-    const F *xb = sm.xs[j & 1];
+    const double tj = sm.tau[j], sj = sm.scal[j];
+    const double *xb = sm.xs[j & 1];
     const int sb = nr.first(), se = nr.end(j);
-    F x[TS];
+    double x[TS];
 #pragma unroll
-    for (int s = 0; s < TS; ++s) x[s] = F(0);
+    for (int s = 0; s < TS; ++s) x[s] = 0.0;
 #pragma unroll
     for (int s = U; s < TS; ++s) {
       if (s >= se) break;
       if (s < sb) continue;
       x[s] = xb[16 * s + rg];
     }
-    F w[TC], sw[TC];
+    double w[TC], sw[TC];
 #pragma unroll
-    for (int t = 0; t < TC; ++t) w[t] = sw[t] = F(0);
-    if (tj != F(0)) {
-      F e[TC];
+    for (int t = 0; t < TC; ++t) w[t] = sw[t] = 0.0;
+    if (tj != 0.0) {
+      double e[TC];
 #pragma unroll
       for (int t = 0; t < TC; ++t) {
-        F acc = F(0);
+        double acc = 0.0;
 #pragma unroll
         for (int s = U; s < TS; ++s) {
           if (s >= se) break;
@@ -214,17 +207,17 @@ __device__ __forceinline__ void qr_block(F (&A)[TS][TC], const NodeRows<MERGE> &
       }
       // what follows from a column's sum -- d_q, w_q and s_j w_q, or Z(q, j)
       // -- is computed on the lane that holds it, once for all TC columns
-      const F sum = half_sum_scatter<TC>(e, rg);
+      const double sum = half_sum_scatter<TC>(e, rg);
       const int ts = sum_index<TC>(rg), qs = cg + 16 * ts;
-      F ajq = F(0);
+      double ajq = 0.0;
 #pragma unroll
       for (int t = 0; t < TC; ++t) {
-        const F v = __shfl_sync(0xffffffffu, A[U][t], jr, 16);
+        const double v = __shfl_sync(0xffffffffu, A[U][t], jr, 16);
         ajq = (t == ts) ? v : ajq;
       }
-      const F d = fma(sj, sum, ajq);
-      const F wq = qs > j ? tj * d : F(0);
-      const F swq = sj * wq;
+      const double d = fma(sj, sum, ajq);
+      const double wq = qs > j ? tj * d : 0.0;
+      const double swq = sj * wq;
       if (qs < j && rg == sum_lane<TC>(ts)) sm.Z[j * (j - 1) / 2 + qs] = sm.scal[qs] * d;
 #pragma unroll
       for (int t = U; t < TC; ++t) {
@@ -235,46 +228,46 @@ __device__ __forceinline__ void qr_block(F (&A)[TS][TC], const NodeRows<MERGE> &
 #pragma unroll
       for (int t = 0; t < TC; ++t) {
         const int q = cg + 16 * t;
-        if (q < j) sm.Z[j * (j - 1) / 2 + q] = F(0);
+        if (q < j) sm.Z[j * (j - 1) / 2 + q] = 0.0;
       }
     }
     const bool row_j = rg == jr;
     // the column after j first, then its reflector, then the other columns
-    if (tj != F(0) && cg > jr) update_col<F, TC, TS, U>(A, x, sb, se, U, w[U], sw[U], row_j);
+    if (tj != 0.0 && cg > jr) update_col<TC, TS, U>(A, x, sb, se, U, w[U], sw[U], row_j);
     if (jr == 15) {
       if constexpr (U + 1 < TC) {
-        if (tj != F(0)) update_col<F, TC, TS, U>(A, x, sb, se, U + 1, w[U + 1], sw[U + 1], row_j);
-        if (j + 1 < kmax && cg == 0) reflect<F, TC, TS, U + 1, MERGE>(A, nr, rg, 0, j + 1, sm.xs[(j + 1) & 1], sm.tau, sm.scal);
+        if (tj != 0.0) update_col<TC, TS, U>(A, x, sb, se, U + 1, w[U + 1], sw[U + 1], row_j);
+        if (j + 1 < kmax && cg == 0) reflect<TC, TS, U + 1, MERGE>(A, nr, rg, 0, j + 1, sm.xs[(j + 1) & 1], sm.tau, sm.scal);
 #pragma unroll
         for (int t = U + 2; t < TC; ++t)
-          if (tj != F(0)) update_col<F, TC, TS, U>(A, x, sb, se, t, w[t], sw[t], row_j);
+          if (tj != 0.0) update_col<TC, TS, U>(A, x, sb, se, t, w[t], sw[t], row_j);
       }
     } else {
-      if (j + 1 < kmax && cg == jr + 1) reflect<F, TC, TS, U, MERGE>(A, nr, rg, jr + 1, j + 1, sm.xs[(j + 1) & 1], sm.tau, sm.scal);
+      if (j + 1 < kmax && cg == jr + 1) reflect<TC, TS, U, MERGE>(A, nr, rg, jr + 1, j + 1, sm.xs[(j + 1) & 1], sm.tau, sm.scal);
 #pragma unroll
       for (int t = U + 1; t < TC; ++t)
-        if (tj != F(0)) update_col<F, TC, TS, U>(A, x, sb, se, t, w[t], sw[t], row_j);
+        if (tj != 0.0) update_col<TC, TS, U>(A, x, sb, se, t, w[t], sw[t], row_j);
     }
   }
 }
 
-template <class F, int TC, int TS, int U, bool MERGE>
-__device__ __forceinline__ void qr_blocks(F (&A)[TS][TC], const NodeRows<MERGE> &nr, RegSmem<F, TC, TS> &sm,
+template <int TC, int TS, int U, bool MERGE>
+__device__ __forceinline__ void qr_blocks(double (&A)[TS][TC], const NodeRows<MERGE> &nr, RegSmem<TC, TS> &sm,
                                           int rg, int cg, int kmax) {
   if constexpr (U < TC) {
-    qr_block<F, TC, TS, U, MERGE>(A, nr, sm, rg, cg, kmax);
-    qr_blocks<F, TC, TS, U + 1, MERGE>(A, nr, sm, rg, cg, kmax);
+    qr_block<TC, TS, U, MERGE>(A, nr, sm, rg, cg, kmax);
+    qr_blocks<TC, TS, U + 1, MERGE>(A, nr, sm, rg, cg, kmax);
   }
 }
 
 // The whole node: reflectors, v = s x below the diagonal, T (strict upper part
 // in sm.T, diagonal in sm.tau).  Every thread of the CTA calls it.
-template <class F, int TC, int TS, bool MERGE>
-__device__ __forceinline__ void qr_node(F (&A)[TS][TC], const NodeRows<MERGE> &nr, RegSmem<F, TC, TS> &sm, int kmax) {
+template <int TC, int TS, bool MERGE>
+__device__ __forceinline__ void qr_node(double (&A)[TS][TC], const NodeRows<MERGE> &nr, RegSmem<TC, TS> &sm, int kmax) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int rg = lane & 15, cg = 2 * (tid >> 5) + (lane >> 4);
-  if (kmax > 0 && cg == 0) reflect<F, TC, TS, 0, MERGE>(A, nr, rg, 0, 0, sm.xs[0], sm.tau, sm.scal);
-  qr_blocks<F, TC, TS, 0, MERGE>(A, nr, sm, rg, cg, kmax);
+  if (kmax > 0 && cg == 0) reflect<TC, TS, 0, MERGE>(A, nr, rg, 0, 0, sm.xs[0], sm.tau, sm.scal);
+  qr_blocks<TC, TS, 0, MERGE>(A, nr, sm, rg, cg, kmax);
   __syncthreads();  // every tau, s and Z entry is written
 
   // v = s x below the diagonal of every reflector column
@@ -282,7 +275,7 @@ __device__ __forceinline__ void qr_node(F (&A)[TS][TC], const NodeRows<MERGE> &n
   for (int t = 0; t < TC; ++t) {
     const int q = cg + 16 * t;
     if (q < kmax) {
-      const F sq = sm.scal[q];
+      const double sq = sm.scal[q];
 #pragma unroll
       for (int s = 0; s < TS; ++s)
         if (rg + 16 * s > q) A[s][t] *= sq;
@@ -293,16 +286,16 @@ __device__ __forceinline__ void qr_node(F (&A)[TS][TC], const NodeRows<MERGE> &n
   //      T(j, j) = tau_j; four threads per row i, each over every fourth q
   const int i = tid >> 2, part = tid & 3;
   for (int j = 1; j < kmax; ++j) {
-    const F tj = sm.tau[j];
-    F acc = F(0);
-    if (i < j && tj != F(0))
+    const double tj = sm.tau[j];
+    double acc = 0.0;
+    if (i < j && tj != 0.0)
       for (int q = i + part; q < j; q += 4) {
-        const F tiq = (q == i) ? sm.tau[i] : sm.T[q * (q - 1) / 2 + i];
+        const double tiq = (q == i) ? sm.tau[i] : sm.T[q * (q - 1) / 2 + i];
         acc = fma(tiq, sm.Z[j * (j - 1) / 2 + q], acc);
       }
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-    if (i < j && part == 0) sm.T[j * (j - 1) / 2 + i] = (tj != F(0)) ? -tj * acc : F(0);
+    if (i < j && part == 0) sm.T[j * (j - 1) / 2 + i] = (tj != 0.0) ? -tj * acc : 0.0;
     __syncthreads();  // column j of T is complete before column j + 1 reads it
   }
 }
