@@ -106,7 +106,58 @@ __global__ void __launch_bounds__(256) trsm_diag_kernel(int nb, int nrhs, const 
 }
 
 // ---------------------------------------------------------------------------
-// Few right-hand sides: one cooperative launch, one CTA per diagonal block,
+// One block (n <= kTb), few right-hand sides: substitution with a warp per
+// right-hand side, its elements in registers (row lane + 32 t in x[t]), the
+// triangle in shared memory; x_j goes round by a shuffle, no barrier after the
+// load.  The operations on every element are trsm_diag_kernel's, in its order:
+// a division per element, so that diagonals whose reciprocal is not a finite
+// number are no special case, and the residual of substitution however
+// ill-conditioned the triangle is (the product with an inverse has neither).
+// Bound by the chain of n divisions (436 clocks) for U and multiply-adds for L.
+// ---------------------------------------------------------------------------
+template <bool LOWER, bool UNIT>
+__global__ void __launch_bounds__(512) trsv_block_kernel(int n, int nrhs, const double *T, int ldt, double *B, int ldb,
+                                                         const int *skip) {
+  extern __shared__ __align__(16) double tsm[];  // T(i, j) at i + j (kTb + 1)
+  if (skip && *skip) return;
+  const int lane = threadIdx.x & 31;
+  for (int idx = threadIdx.x; idx < n * n; idx += 512) {
+    const int i = idx % n, j = idx / n;
+    tsm[i + j * (kTb + 1)] = T[i + (size_t)j * ldt];
+  }
+  __syncthreads();
+  for (int c = threadIdx.x >> 5; c < nrhs; c += 16) {
+    double *b = B + (size_t)c * ldb;
+    double x[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) x[t] = lane + 32 * t < n ? b[lane + 32 * t] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int s = LOWER ? u : 3 - u;
+#pragma unroll 1
+      for (int q = 0; q < 32; ++q) {
+        const int jl = LOWER ? q : 31 - q, j = 32 * s + jl;
+        if (j >= n) continue;
+        const double *tj = tsm + j * (kTb + 1);
+        double xj = __shfl_sync(0xffffffffu, x[s], jl);
+        if (!UNIT) xj = xj / tj[j];
+        if (lane == jl) x[s] = xj;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int t = LOWER ? s + v : s - v, i = lane + 32 * t;
+          if (t < 0 || t > 3) continue;
+          if (LOWER ? i > j && i < n : i < j) x[t] = fma(-tj[i], xj, x[t]);
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (lane + 32 * t < n) b[lane + 32 * t] = x[t];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Few right-hand sides, several blocks: one cooperative launch, one CTA per diagonal block,
 // ordered by per-block ready flags instead of grid-wide barriers.
 //   Phase 0: CTA c loads diagonal block c of T and inverts its four 32 x 32
 //            diagonal sub-blocks, one warp each (one per SM sub-partition; a
@@ -369,7 +420,7 @@ static cudaError_t trsm_left_flags(bool lower, bool unit, int n, int nrhs, const
   });
   if (e != cudaSuccess) return e;
   const int nblk = (n + TB - 1) / TB;
-  if (nblk > 1 && (e = cudaMemsetAsync(ws.flags, 0, (size_t)nblk, st)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(ws.flags, 0, (size_t)nblk, st)) != cudaSuccess) return e;
   FlagArgs fa;
   fa.flags = ws.flags;
   fa.status = status;
@@ -382,8 +433,21 @@ static cudaError_t trsm_left_flags(bool lower, bool unit, int n, int nrhs, const
   void *args[] = {&n, &nrhs, (void *)&T, &ldt, &B, &ldb, &un, &fa};
   void *fn = lower ? (void *)trsv_flag_kernel<true, TB> : (void *)trsv_flag_kernel<false, TB>;
   ProfScope ps(kClsSolve, st, (double)n * n * nrhs);
-  if (nblk == 1) return cudaLaunchKernel(fn, dim3(1), dim3(256), args, smem, st);  // waits for nobody
   return cudaLaunchCooperativeKernel(fn, dim3(nblk), dim3(256), args, smem, st);
+}
+
+template <bool LOWER, bool UNIT>
+static cudaError_t trsv_block(int n, int nrhs, const double *T, int ldt, double *B, int ldb, const int *skip,
+                              cudaStream_t st) {
+  static std::atomic<unsigned long long> init{0};
+  cudaError_t e = once_per_device(init, [] {
+    return cudaFuncSetAttribute(trsv_block_kernel<LOWER, UNIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kTb * (kTb + 1) * 8);
+  });
+  if (e != cudaSuccess) return e;
+  ProfScope ps(kClsSolve, st, (double)n * n * nrhs);
+  trsv_block_kernel<LOWER, UNIT><<<1, 512, (size_t)n * (kTb + 1) * 8, st>>>(n, nrhs, T, ldt, B, ldb, skip);
+  return cudaGetLastError();
 }
 
 cudaError_t trsm_left(bool lower, bool unit, int n, int nrhs, const double *T, int ldt, double *B, int ldb,
@@ -393,10 +457,12 @@ cudaError_t trsm_left(bool lower, bool unit, int n, int nrhs, const double *T, i
   // Blocks of 64 rows while there is an SM for each: the chain is one block
   // product and one block solve per block on a single SM's FP64 pipe, so twice
   // the blocks of a quarter the work each (order 2048, 4 right-hand sides: 925
-  // us a triangle before, 750 with blocks of 128, 440 with 64).  A single block
-  // of up to 128 rows has no chain.
+  // us a triangle before, 750 with blocks of 128, 440 with 64).
+  if (nrhs <= kCoopMaxRhs && n <= kTb)
+    return !lower ? (unit ? trsv_block<false, true> : trsv_block<false, false>)(n, nrhs, T, ldt, B, ldb, skip, st)
+                  : (unit ? trsv_block<true, true> : trsv_block<true, false>)(n, nrhs, T, ldt, B, ldb, skip, st);
   if (nrhs <= kCoopMaxRhs && n <= coop_max_n()) {
-    if (n > kTb && n <= coop_max_n() / 2)
+    if (n <= coop_max_n() / 2)
       return trsm_left_flags<64>(lower, unit, n, nrhs, T, ldt, B, ldb, ws, status, status_bit, skip, st);
     return trsm_left_flags<kTb>(lower, unit, n, nrhs, T, ldt, B, ldb, ws, status, status_bit, skip, st);
   }
