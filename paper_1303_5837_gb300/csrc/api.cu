@@ -271,7 +271,7 @@ int caqr_run(int m, int n, double *A, int lda, int b, const ca_tree_t *tree, dou
                                 dev_info + 1, stream);
       if (f64ws && tree_tc_pays(mk, bk, ncols, L, plan))
         return tree_apply_qt_tc(mk, bk, b, P, lda, L, plan, Tp, C, lda, ncols, ws, f64ws, kTcF64Slices, 1,
-                                dev_info + 1, stream, 1);
+                                dev_info + 1, stream, kTreeKeep);
       return tree_apply_qt(mk, bk, b, P, lda, L, plan, Tp, C, lda, ncols, ws, stream);
     };
     if (nt > 0) {
@@ -305,7 +305,7 @@ cudaError_t getrs_run(int n, int nrhs, const double *LU, int lda, const int *ipi
 size_t qr_f64_ws_bytes(int m, int n, int b, const ca_tree_t *tree, int nl) {
   Plan plan;
   if (b >= n || !build_plan(nl, *tree, plan) || !tree_tc_pays(m, b, n - b, tree->leaf_rows, plan)) return 0;
-  return tree_tc_ws_bytes(m, b, n - b, tree->leaf_rows, nl, kTcF64Slices);
+  return tree_tc_ws_bytes(m, b, n - b, tree->leaf_rows, nl, kTcF64Slices, true);
 }
 
 size_t caqr_mixed_ws(int m, int n, int b, const ca_tree_t *tree, int nl, int slices) {

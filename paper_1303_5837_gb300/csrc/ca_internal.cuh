@@ -310,18 +310,19 @@ struct TcGemm {
   double sign;
   int S, exact;
   const int *skip;      // as for the LU launchers (null: always run)
-  // full: the result stands in for an FP64 product.  Vectors whose digits
-  // cannot (a value that is not finite, or a largest magnitude near the ends
-  // of the range) are multiplied in FP64 by the epilogue.  kexp: A's column k
-  // is taken times 2^-kexp[k] and B's row k times 2^kexp[k] (exact; null: 0).
-  // reuse_a: A's digits of the previous call with this workspace, A and kexp
-  // are still in place.
-  int full;
+  // keep > 0 (7 exact digits): the result stands in for an FP64 product.
+  // Elements with |C_ij| + sum_k |a_ik| |b_kj| below keep times the powers of
+  // two above their vectors' largest magnitudes, and those of vectors with
+  // values that are not finite or near the ends of the range, are multiplied
+  // in FP64 (tc_check_kernel).  kexp: A's column k is taken times 2^-kexp[k]
+  // and B's row k times 2^kexp[k] (exact; null: 0).  reuse_a: A's digits of
+  // the previous call with this workspace, A and kexp are still in place.
+  float keep;
   const int *kexp;
   int reuse_a;
 };
 cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st);
-size_t tc_gemm_ws_bytes_batched(int m, int n, int k, int S, int nbatch);
+size_t tc_gemm_ws_bytes_batched(int m, int n, int k, int S, int nbatch, bool keep = false);
 size_t tc_gemm_ws_bytes(int m, int n, int k, int S);
 bool tc_gemm_supported(int k, int S, int exact);
 cudaError_t gemm_minus_tc(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C,
@@ -337,11 +338,12 @@ cudaError_t gemm_minus_f64_tc(int m, int n, int k, const double *A, int lda, con
                               int ldc, bool first, void *ws, int *status, cudaStream_t st, const int *skip);
 
 // CAQR tree update on the tensor cores (update_tc.cu)
-size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, int S);
+size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, int S, bool keep = false);
 cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, int leaf_rows, const Plan &plan,
                              const double *Tp, double *C, int ldc, int ncols, const QrPanelWs &ws, void *tcws,
-                             int S, int exact, int *status, cudaStream_t st, int full = 0);
-// whether the FP64 update (7 exact digits, full = 1) is faster there than on
+                             int S, int exact, int *status, cudaStream_t st, float keep = 0.0f);
+constexpr float kTreeKeep = 1.0f / 32;  // TcGemm::keep of the FP64 tree update (update_tc.cu)
+// whether the FP64 update (7 exact digits, keep > 0) is faster there than on
 // the FP64 pipe
 bool tree_tc_pays(int mk, int bk, int ncols, int leaf_rows, const Plan &plan);
 

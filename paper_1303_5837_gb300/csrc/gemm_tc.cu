@@ -135,6 +135,21 @@ __device__ __forceinline__ void tmem_ld_32x4(uint32_t taddr, uint32_t (&r)[4]) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 }
+// 32 TMEM lanes x 32 consecutive 32-bit columns, with the wait
+__device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+}
 // waits for the loads; every value passes through, so that no use of it moves up
 __device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[8][4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
@@ -321,11 +336,13 @@ struct TcArgs {
   int sign;            // C -= sign * A B, sign = +1 or -1
   int *status;
   const int *skip;     // nonzero: a stage enqueued ahead that is not needed, do nothing
-  int full;            // vectors marked kExOdd are multiplied in FP64 from A and B
+  int slices;          // operand slices per item: S digits, then the magnitudes when keep > 0
+  float keep;          // TcGemm::keep
+  unsigned *fp64;      // keep > 0: bit c of word [item][row / 32][column / 32]: these 32 rows of column c take FP64
   TcOperand A, B;
 };
 
-// Exponent mark of a vector that has no digits (TcGemm::full).
+// Exponent mark of a vector that has no digits (TcGemm::keep).
 constexpr int kExOdd = 1 << 20;
 
 // Element (v, k) of item b of an operand, 0 outside its structure.
@@ -342,17 +359,76 @@ __device__ __forceinline__ int operand_k(const TcOperand &o, int b, bool last) {
   return o.K_item ? o.K_item[b] : (last ? o.K_last : o.K);
 }
 
-// c - sign sum_k A(i, k) B(k, j) as a chain of FP64 multiply-adds: the
-// elements whose row or column has no digits.
-__device__ __noinline__ double odd_element(const TcArgs &a, int item, int i, int j, double c) {
+// C -= sign A B in FP64 for the columns n0 + c, bit c of `cols`, of the rows
+// r0 .. r0 + 31: what the digits cannot stand for.  A chain of multiply-adds
+// over k, then one subtraction, as in gemm_fp64.cu (the same bits).  The whole
+// CTA calls it; a warp takes every eighth column, a lane a row, so that the
+// usual one or two columns cost one chain of K multiply-adds (64 clocks of the
+// FP64 pipe each, 4 us) and not the 32 us of all 32 columns.  All of K is
+// staged at once (sm: 2 x 128 x 33 doubles; K <= 128).
+constexpr int kFpLd = 33;
+
+__device__ __noinline__ void fp64_block(const TcArgs &a, int item, int r0, int n0, unsigned cols, int mv, int nvv,
+                                        double *Cb, double *sm) {
+  __shared__ int list[32];  // the columns
   const bool last = item == a.nbatch - 1;
   const int K = min(operand_k(a.A, item, last), operand_k(a.B, item, last));
   const double *X = operand_item(a.A, item), *Y = operand_item(a.B, item);
-  for (int k = 0; k < K; ++k) {
-    const double x = operand_at(a.A, X, i, k);
-    c = fma(a.sign > 0 ? -x : x, operand_at(a.B, Y, j, k), c);
+  double *As = sm, *Bs = sm + 128 * kFpLd;  // (k, row) and (k, place in the list)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nf = __popc(cols);
+  __syncthreads();  // the operands of an earlier call have been read
+  if (tid < 32 && (cols >> tid & 1u)) list[__popc(cols & ((1u << tid) - 1u))] = tid;
+  __syncthreads();
+  // what A's structure leaves of k for these rows
+  int klo = 0, khi = K;
+  if (a.A.shape == 1) {
+    if (a.A.trans)
+      klo = max(0, r0 - a.A.roff);
+    else
+      khi = min(K, r0 + 32 + a.A.roff);
+  } else if (a.A.shape == 2) {
+    if (a.A.trans)
+      khi = min(K, r0 + 32 - a.A.roff);
+    else
+      klo = max(0, r0 + a.A.roff);
   }
-  return c;
+  const int kr = max(0, khi - klo);
+#pragma unroll 8
+  for (int e = tid; e < 32 * kr; e += 256) {  // along A's contiguous index
+    const int v = a.A.sv == 1 ? e & 31 : e / kr, k = a.A.sv == 1 ? e >> 5 : e % kr;
+    As[k * kFpLd + v] = r0 + v < mv ? operand_at(a.A, X, r0 + v, klo + k) : 0.0;
+  }
+#pragma unroll 4
+  for (int e = tid; e < nf * kr; e += 256) {
+    const int v = e / kr, k = e % kr, c = n0 + list[v];
+    Bs[k * kFpLd + v] = c < nvv ? operand_at(a.B, Y, c, klo + k) : 0.0;
+  }
+  __syncthreads();
+  const int nv = (nf - warp + 7) / 8;  // this warp's columns
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int k = 0; k < kr; ++k) {
+    const double x = As[k * kFpLd + lane];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      if (v >= nv) break;
+      acc[v] = fma(x, Bs[k * kFpLd + warp + 8 * v], acc[v]);
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    if (v >= nv) break;
+    const int c = n0 + list[warp + 8 * v];
+    if (r0 + lane >= mv || c >= nvv) continue;
+    double *p = Cb + r0 + lane + (size_t)c * a.ldc;
+    *p = a.sign > 0 ? *p - acc[v] : *p + acc[v];
+  }
+}
+
+__device__ __forceinline__ unsigned *fp64_word_at(const TcArgs &a, int item, int mtile, int quad, int n0) {
+  return a.fp64 + (((size_t)item * (a.mpad / kTcBM) + mtile) * 4 + quad) * (a.npad / 32) + n0 / 32;
+}
+__device__ __forceinline__ unsigned fp64_word(const TcArgs &a, int item, int mtile, int quad, int n0) {
+  return a.keep > 0.0f ? *fp64_word_at(a, item, mtile, quad, n0) : 0u;
 }
 
 // Operand tiles for one K block: S boxes of A digits (128 x bk) then S boxes
@@ -363,7 +439,7 @@ __host__ __device__ inline size_t tc_stage_bytes(int S, int bn, int bk) {
 
 __global__ void __launch_bounds__(256, 2)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-                   TcArgs a) {
+                   const __grid_constant__ TcArgs a) {
   extern __shared__ uint8_t smem_raw[];
   if (a.skip && *a.skip) return;  // before any barrier, copy or tensor-memory allocation
   uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -382,6 +458,8 @@ __global__ void __launch_bounds__(256, 2)
   const int mv = a.m_item ? a.m_item[item] : (last ? a.m_last : a.m);
   const int nvv = a.n_item ? a.n_item[item] : (last ? a.n_last : a.n);
   if (m0 >= mv || n0 >= nvv) return;  // an empty tile of a short batch item (uniform per CTA)
+  __shared__ unsigned other_of[4];    // per 32 rows: the columns left to fp64_block
+  if (threadIdx.x < 4) other_of[threadIdx.x] = fp64_word(a, item, blockIdx.x, threadIdx.x, n0);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -416,8 +494,8 @@ __global__ void __launch_bounds__(256, 2)
       uint8_t *sb = sa + (size_t)a.S * boxA;
       mbar_expect_tx(&full[st], (uint32_t)stage_bytes);
       for (int s = 0; s < a.S; ++s) {
-        tma_load_2d(sa + (size_t)s * boxA, &mapA, &full[st], kb * a.bk, (item * a.S + s) * a.mpad + m0);
-        tma_load_2d(sb + (size_t)s * boxB, &mapB, &full[st], kb * a.bk, (item * a.S + s) * a.npad + n0);
+        tma_load_2d(sa + (size_t)s * boxA, &mapA, &full[st], kb * a.bk, (item * a.slices + s) * a.mpad + m0);
+        tma_load_2d(sb + (size_t)s * boxB, &mapB, &full[st], kb * a.bk, (item * a.slices + s) * a.npad + n0);
       }
       if (st == 0)
         ++issued0;
@@ -502,6 +580,7 @@ __global__ void __launch_bounds__(256, 2)
     const int er = rin ? a.ea[(size_t)item * a.mpad + row] : 0;
     const int *ebi = a.eb + (size_t)item * a.npad;
     double *Cb = a.C + (size_t)item * a.sbc + (a.coff ? a.coff[item] : 0);
+    const unsigned other = other_of[quad];
     // exact mode: the digit diagonals D = 0 .. S-1 (weights 2^(-8 D)) are
     // integers below 2^24; combine them in integer arithmetic,
     //   T_hi = sum_{D <= 4} acc_D 2^(8 (4 - D)),  T_lo = sum_{D > 4} acc_D 2^(8 (6 - D)),
@@ -558,7 +637,7 @@ __global__ void __launch_bounds__(256, 2)
           }
           bool sl;
           cv[j] -= nacc > 5 ? scaled_sum_rn(hi[j], lo[j], sc - 48, sl) : scaled_rn(hi[j], sc - 32, sl);
-          slow |= (sl || (a.full && sc > kExOdd / 2)) ? 1u << j : 0u;
+          slow |= sl ? 1u << j : 0u;
         } else {
           cv[j] = fma((double)(-a.sign * __uint_as_float(r[0][j])), pow2i(sc), cv[j]);
         }
@@ -570,14 +649,13 @@ __global__ void __launch_bounds__(256, 2)
           if (!((slow >> j) & 1u) || !rin || col >= nvv) continue;
           const int sc = er + ec[j] - 16;
           const double c = __ldcg(Cb + row + (size_t)col * a.ldc);
-          cv[j] = (a.full && sc > kExOdd / 2) ? odd_element(a, item, row, col, c)
-                                              : c - scaled_sum_slow(hi[j], lo[j], sc - 48);
+          cv[j] = c - scaled_sum_slow(hi[j], lo[j], sc - 48);
         }
       }
 #pragma unroll
       for (int j = 0; j < kEp; ++j) {
         const int col = n0 + c0 + j;
-        if (rin && col < nvv) Cb[row + (size_t)col * a.ldc] = cv[j];
+        if (rin && col < nvv && !((other >> (c0 + j)) & 1u)) Cb[row + (size_t)col * a.ldc] = cv[j];
       }
     }
   }
@@ -590,6 +668,119 @@ __global__ void __launch_bounds__(256, 2)
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, (uint32_t)a.tmem_cols);
+  // (the operand stages are free: every copy has landed, every MMA is done)
+  for (int q = 0; q < 4; ++q)
+    if (other_of[q])
+      fp64_block(a, item, m0 + 32 * q, n0, other_of[q], mv, nvv,
+                 a.C + (size_t)item * a.sbc + (a.coff ? a.coff[item] : 0), reinterpret_cast<double *>(base));
+}
+
+// --------------------------------------------------------------------------
+// Where the digits may stand in for FP64 (TcGemm::keep).  The digits hold an
+// operand to 2^-57 of its vector's 2^e > max, so an element's error is up to
+// 2.5 K 2^-56 2^(e_i + f_j) (representation 2 K 2^-57, dropped products k + l
+// >= 9 6 K 2^-58) however small the element is, while FP64 multiply-adds have
+// the bound K 2^-53 (|C_ij| + sum_k |a_ik| |b_kj|).  The first is below the
+// second where
+//   |C_ij| + sum_k |a_ik| |b_kj| >= keep 2^(e_i + f_j),  keep = 2.5 / 8.
+// This kernel checks that for every element: one bf16 MMA product of the
+// operands' magnitudes (rounded down, relative to 2^e; a nonzero one is at
+// least 2^-40) per 128 x 128 tile, C only where the sum alone does not reach
+// keep.  A sum of zero means that every product is zero: no error.  Columns
+// with an element that fails take FP64 in the 32 rows that hold it, which
+// depends on nothing but those rows and that column: the result does not
+// change with the way a matrix is cut into calls.  Non-finite vectors and
+// those with values near the ends of the range (kExOdd) take it too.
+// Bound by its launch and the chain load - MMA - read for small updates, by the
+// operands' L2 reads for large ones: CALU + solve of n = 10240 113.4 -> 114.5
+// ms (no element fails there), CAQR + solve of n = 6144 128.2 -> 146.0 ms
+// (1335 checks of about 15 us; 6 % of the updates' blocks of 32 x 32 hold an
+// element that fails, mostly in T^T W, 2 % of their columns).
+// --------------------------------------------------------------------------
+constexpr int kChkN = 128;
+
+__global__ void __launch_bounds__(256, 3)
+    tc_check_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                    const __grid_constant__ TcArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  if (a.skip && *a.skip) return;
+  uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  __shared__ uint64_t bars[3];  // [0], [1]: a 64-wide half of K has arrived; [2]: the MMAs are done
+  __shared__ uint32_t tslot;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int m0 = blockIdx.x * kTcBM, n0 = blockIdx.y * kChkN;
+  const int item = blockIdx.z;
+  const bool last = item == a.nbatch - 1;
+  const int mv = a.m_item ? a.m_item[item] : (last ? a.m_last : a.m);
+  const int nvv = a.n_item ? a.n_item[item] : (last ? a.n_last : a.n);
+  if (m0 >= mv || n0 >= nvv) return;
+  constexpr int boxA = kTcBM * 64 * 2, boxB = kChkN * 64 * 2;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 3; ++i) mbar_init(&bars[i], 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) {
+    tmem_alloc(&tslot, kChkN);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tslot;
+  if (warp == 0 && elect_one()) {
+    for (int kb = 0; kb < a.kblocks; ++kb) {  // at most two: all of K is resident
+      uint8_t *sa = base + kb * (boxA + boxB);
+      mbar_expect_tx(&bars[kb], boxA + boxB);
+      tma_load_2d(sa, &mapA, &bars[kb], kb * 64, (item * a.slices + a.S) * a.mpad + m0);
+      tma_load_2d(sa + boxA, &mapB, &bars[kb], kb * 64, (item * a.slices + a.S) * a.npad + n0);
+    }
+  } else if (warp == 1 && elect_one()) {
+    for (int kb = 0; kb < a.kblocks; ++kb) {
+      if (!mbar_wait(&bars[kb], 0, kWaitLimit)) {
+        atomicOr(a.status, 4);
+        break;
+      }
+      tc_fence_after();
+      const uint8_t *sa = base + kb * (boxA + boxB);
+      const uint64_t ad = sw_desc(smem_u32(sa), 2), bd = sw_desc(smem_u32(sa + boxA), 2);
+      for (int ks = 0; ks < 4; ++ks)
+        tc_mma(tmem, ad + 2 * ks, bd + 2 * ks, idesc_bf16_f32(kTcBM, kChkN), kb > 0 || ks > 0);
+    }
+    tc_commit(&bars[2]);
+  }
+  __syncthreads();
+  bool ok = mbar_wait(&bars[2], 0, kWaitLimit);
+  for (int kb = 0; kb < a.kblocks; ++kb) ok &= mbar_wait(&bars[kb], 0, kWaitLimit);  // its copies have landed
+  if (!ok && lane == 0) atomicOr(a.status, 8);
+  tc_fence_after();
+  const int quad = warp & 3, half = warp >> 2;
+  const int row = m0 + 32 * quad + lane;
+  const bool rin = row < mv;
+  const int er = rin ? a.ea[(size_t)item * a.mpad + row] : 0;
+  const double *Cb = a.C + (size_t)item * a.sbc + (a.coff ? a.coff[item] : 0);
+  for (int c0 = half * 64; c0 < half * 64 + 64 && n0 + c0 < nvv; c0 += 32) {
+    uint32_t r[32];
+    tmem_ld_32x32(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0, r);
+    const int mycol = n0 + c0 + lane;
+    const int myec = mycol < nvv ? a.eb[(size_t)item * a.npad + mycol] : 0;
+    unsigned fail = __ballot_sync(0xffffffffu, myec > kExOdd / 2);
+    if (er > kExOdd / 2 || !ok) fail = 0xffffffffu;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      const float v = __uint_as_float(r[c]);
+      const int ec = __shfl_sync(0xffffffffu, myec, c);
+      if (v < a.keep && v != 0.0f && !((fail >> c) & 1u)) {
+        // rin and the column is valid: padding has no magnitudes
+        const double lack = (double)(a.keep - v) * pow2i(er + ec);
+        if (er + ec > 1000 || !(fabs(Cb[row + (size_t)(n0 + c0 + c) * a.ldc]) >= lack)) fail |= 1u << c;
+      }
+    }
+    fail = __reduce_or_sync(0xffffffffu, rin ? fail : 0u);
+    if (lane == 0) *fp64_word_at(a, item, blockIdx.x, quad, n0 + c0) = fail;
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, kChkN);
 }
 
 // --------------------------------------------------------------------------
@@ -599,15 +790,31 @@ __global__ void __launch_bounds__(256, 2)
 // the structure rule on (r, q) = (row, column) of the source:
 // shape 0 dense, 1 unit lower (r > q stored, r == q is one, r < q zero),
 // 2 upper (r <= q stored); (r, q) = (v + roff, k) or, transposed, (k + roff, v).
-// Output: out[((b * S + s) * vpad + v) * kpad + k], exponent ex[b * vpad + v].
+// Output: out[((b * slices + s) * vpad + v) * kpad + k], exponent ex[b * vpad + v];
+// slices = S, with KEEP one more: the magnitudes |x| 2^-e rounded down.
 // --------------------------------------------------------------------------
-template <bool FULL, int S>
-__global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int vpad, int kpad, int exact,
-                                                    __nv_bfloat16 *__restrict__ out, int *__restrict__ ex,
-                                                    const int *skip, const int *kexp, int ksign) {
+// One launch splits both operands: blocks from nblkA on work on B.
+struct SplitSide {
+  TcOperand o;
+  int vpad;
+  __nv_bfloat16 *out;
+  int *ex;
+  int ksign;           // KEEP: kexp is taken with this sign
+};
+
+template <bool KEEP, int S>
+__global__ void __launch_bounds__(256) split_kernel(const __grid_constant__ SplitSide sideA,
+                                                    const __grid_constant__ SplitSide sideB, int nblkA, int nbatch,
+                                                    int kpad, int exact, const int *skip, const int *kexp) {
   if (skip && *skip) return;
+  const bool second = (int)blockIdx.x >= nblkA;
+  const SplitSide &d = second ? sideB : sideA;
+  const TcOperand &o = d.o;
+  const int vpad = d.vpad, ksign = d.ksign;
+  __nv_bfloat16 *__restrict__ out = d.out;
+  int *__restrict__ ex = d.ex;
   const int lane = threadIdx.x & 31;
-  const int v = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int v = ((int)blockIdx.x - (second ? nblkA : 0)) * 8 + (threadIdx.x >> 5);
   const int b = blockIdx.y;
   if (v >= vpad) return;
   const bool last = b == nbatch - 1;
@@ -615,6 +822,7 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
   const int K = operand_k(o, b, last);
   const double *X = operand_item(o, b);
   constexpr int kPer = 8;  // K <= 256
+  constexpr int kSlices = S + (KEEP ? 1 : 0);
   double x[kPer];
   int sh[kPer];            // the element is taken times 2^sh
   unsigned long long mx = 0;
@@ -629,10 +837,10 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
     const unsigned long long bits = absbits(val);
     mx = bits > mx ? bits : mx;
     sh[t] = 0;
-    if constexpr (FULL) {
+    if constexpr (KEEP) {
       if (kexp && k < K) sh[t] = ksign * kexp[k];
       if (bits != 0) me = max(me, (int)(bits >> 52) + sh[t]);
-      odd |= (bits >> 52) == 0x7ffull;
+      odd |= (bits >> 52) == 0x7ffull || ((bits >> 52) == 0 && bits != 0);  // (the digits drop subnormals)
     }
   }
 #pragma unroll
@@ -646,12 +854,12 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
     const int E = (int)(mx >> 52);
     e = (E == 0) ? -1021 : E - 1022;
   }
-  if constexpr (FULL) {
+  if constexpr (KEEP) {
     me = __reduce_max_sync(0xffffffffu, me);
     odd = __reduce_or_sync(0xffffffffu, odd);
     if (mx != 0) {
       e = me - 1022;
-      if (odd || e < -900 || e > 1000) {  // no digits: FP64 in the epilogue
+      if (odd || e < -900 || e > 1000) {  // no digits: FP64
         e = kExOdd;
 #pragma unroll
         for (int t = 0; t < kPer; ++t) x[t] = 0.0;
@@ -669,7 +877,7 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
     // is d_0.  A byte becomes a float by putting it into the mantissa of 2^23
     // (no conversion instruction).
     constexpr unsigned long long bias = 0x0080808080808080ull & ((1ull << (8 * (S - 1))) - 1);
-    const unsigned long long F = (unsigned long long)fixed_point_digits(x[t], FULL ? e - sh[t] : e, S) + bias;
+    const unsigned long long F = (unsigned long long)fixed_point_digits(x[t], KEEP ? e - sh[t] : e, S) + bias;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       const int sft = 8 * (S - 1 - s);
@@ -678,7 +886,14 @@ __global__ void __launch_bounds__(256) split_kernel(TcOperand o, int nbatch, int
       // stored value: d_s (exact mode) or d_s 2^(-8 s) (fused mode), exact in bf16
       // 2^(-8 s) as a float from its exponent field (s <= 7: a normal number)
       const float w = exact ? 1.0f : __int_as_float((127 - 8 * s) << 23);
-      out[(((long long)b * S + s) * vpad + v) * kpad + k] = __float2bfloat16_rn(d * w);
+      out[(((long long)b * kSlices + s) * vpad + v) * kpad + k] = __float2bfloat16_rn(d * w);
+    }
+    if constexpr (KEEP) {
+      const unsigned long long bits = absbits(x[t]);
+      const int ed = (int)(bits >> 52) - 1023 + sh[t] - e;  // below 0; a subnormal's is not used
+      const unsigned m = bits == 0 ? 0u : ed < -40 || (bits >> 52) == 0 ? (127u - 40u) << 7
+                                                    : ((unsigned)(127 + ed) << 7) | (unsigned)((bits >> 45) & 0x7f);
+      out[(((long long)b * kSlices + S) * vpad + v) * kpad + k] = __ushort_as_bfloat16((unsigned short)m);
     }
   }
 }
@@ -786,11 +1001,12 @@ static bool tc_config(int S, int exact, int kpad, TcCfg &c) {
   return false;
 }
 
-size_t tc_gemm_ws_bytes_batched(int m, int n, int k, int S, int nbatch) {
+size_t tc_gemm_ws_bytes_batched(int m, int n, int k, int S, int nbatch, bool keep) {
   const size_t mp = rup(m > 0 ? m : 1, kTcBM), np = rup(n > 0 ? n : 1, 128), kp = rup(k > 0 ? k : 1, kTcKpad);
   const size_t nb = nbatch > 0 ? nbatch : 1;
-  return align256(nb * S * mp * kp * 2) + align256(nb * S * np * kp * 2) + align256(nb * mp * 4) +
-         align256(nb * np * 4) + 256;
+  const size_t ns = S + (keep ? 1 : 0);
+  return align256(nb * ns * mp * kp * 2) + align256(nb * ns * np * kp * 2) + align256(nb * mp * 4) +
+         align256(nb * np * 4) + (keep ? align256(nb * (mp / 32) * (np / 32) * 4) : 0) + 256;
 }
 
 size_t tc_gemm_ws_bytes(int m, int n, int k, int S) { return tc_gemm_ws_bytes_batched(m, n, k, S, 1); }
@@ -811,24 +1027,29 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
   TcCfg cfg;
   if (!tc_config(S, exact, kp, cfg)) return cudaErrorInvalidValue;
   const int bn = cfg.bn;
-  const size_t nb = g.nbatch;
+  const bool keep = g.keep > 0.0f;
+  if (keep && (bn != 32 || !exact || S != kTcF64Slices)) return cudaErrorInvalidValue;  // one word of columns per tile
+  const size_t nb = g.nbatch, ns = S + (keep ? 1 : 0);
   char *p = (char *)(((uintptr_t)ws + 255) & ~(uintptr_t)255);
   __nv_bfloat16 *sa = (__nv_bfloat16 *)p;
-  p += align256(nb * S * mp * kp * 2);
+  p += align256(nb * ns * mp * kp * 2);
   int *ea = (int *)p;
   p += align256(nb * mp * 4);
   __nv_bfloat16 *sb = (__nv_bfloat16 *)p;
-  p += align256(nb * S * np * kp * 2);
+  p += align256(nb * ns * np * kp * 2);
   int *eb = (int *)p;
-  auto split = [&](const TcOperand &o, int vpad, __nv_bfloat16 *out, int *ex, int ksign) {
+  p += align256(nb * np * 4);
+  {
     ProfScope ps(kClsSplit, st, 0.0);
-    const dim3 grid((vpad + 7) / 8, g.nbatch);
+    const SplitSide A = {g.A, mp, sa, ea, -1}, B = {g.B, np, sb, eb, 1};
+    const int nblkA = g.reuse_a ? 0 : (mp + 7) / 8;
+    const dim3 grid(nblkA + (np + 7) / 8, g.nbatch);
     auto run = [&](auto slices) {
       constexpr int kS = decltype(slices)::value;
-      if (g.full)
-        split_kernel<true, kS><<<grid, 256, 0, st>>>(o, g.nbatch, vpad, kp, exact, out, ex, g.skip, g.kexp, ksign);
-      else
-        split_kernel<false, kS><<<grid, 256, 0, st>>>(o, g.nbatch, vpad, kp, exact, out, ex, g.skip, nullptr, 0);
+      if (!keep)
+        split_kernel<false, kS><<<grid, 256, 0, st>>>(A, B, nblkA, g.nbatch, kp, exact, g.skip, nullptr);
+      else if constexpr (kS == kTcF64Slices)
+        split_kernel<true, kS><<<grid, 256, 0, st>>>(A, B, nblkA, g.nbatch, kp, exact, g.skip, g.kexp);
     };
     switch (S) {
       case 1: run(std::integral_constant<int, 1>()); break;
@@ -840,14 +1061,12 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
       case 7: run(std::integral_constant<int, 7>()); break;
       default: run(std::integral_constant<int, 8>()); break;
     }
-  };
-  if (!g.reuse_a) split(g.A, mp, sa, ea, -1);
-  split(g.B, np, sb, eb, 1);
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, sa, kp, (int)(nb * S * mp), kTcBM, cfg.bk) ||
-      !make_map(&mb, sb, kp, (int)(nb * S * np), bn, cfg.bk))
+  if (!make_map(&ma, sa, kp, (int)(nb * ns * mp), kTcBM, cfg.bk) ||
+      !make_map(&mb, sb, kp, (int)(nb * ns * np), bn, cfg.bk))
     return cudaErrorInvalidValue;
   TcArgs a;
   a.kblocks = kp / cfg.bk;
@@ -877,7 +1096,9 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
   a.sign = g.sign > 0 ? 1 : -1;
   a.status = status;
   a.skip = g.skip;
-  a.full = g.full;
+  a.slices = (int)ns;
+  a.keep = g.keep;
+  a.fp64 = (unsigned *)p;
   a.A = g.A;
   a.B = g.B;
   const size_t smem = cfg.smem;
@@ -889,6 +1110,22 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
     return cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   });
   if (e != cudaSuccess) return e;
+  if (keep) {
+    CUtensorMap ca, cb;
+    if (!make_map(&ca, sa, kp, (int)(nb * ns * mp), kTcBM, 64) || !make_map(&cb, sb, kp, (int)(nb * ns * np), kChkN, 64))
+      return cudaErrorInvalidValue;
+    constexpr int kHalfBytes = (kTcBM + kChkN) * 64 * 2;
+    static std::atomic<unsigned long long> cinit{0};
+    e = once_per_device(cinit, [] {
+      return cudaFuncSetAttribute(tc_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kHalfBytes + 1024);
+    });
+    if (e != cudaSuccess) return e;
+    TcArgs c = a;
+    c.kblocks = kp / 64;
+    ProfScope ps(kClsSplit, st, 0.0);
+    tc_check_kernel<<<dim3(mp / kTcBM, np / kChkN, g.nbatch), 256, c.kblocks * kHalfBytes + 1024, st>>>(ca, cb, c);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   dim3 grid(mp / kTcBM, np / bn, g.nbatch);
   // bf16 tensor-core flops issued: S (S + 1) / 2 digit products
   ProfScope ps(kClsGemmTc, st, 2.0 * (double)mp * np * kp * (S * (S + 1) / 2) * nb);
@@ -927,14 +1164,15 @@ cudaError_t gemm_minus_tc(int m, int n, int k, const double *A, int lda, const d
 // --------------------------------------------------------------------------
 // The FP64 Schur update on the tensor cores.  Seven digits of 8 bits hold
 // every operand to 2^-57 of its vector's largest magnitude, the digit sums are
-// exact and C is rounded twice, so the result is closer to the exact product
-// than 128 FP64 multiply-adds, each of which rounds C: relative error 7e-17
-// against 3.8e-16 (256 x 256 x 128, N(0,1)), backward error of the whole CALU
-// 5.6e-15 against 1.2e-14 (n = 2048, N(0,1)).  What the digits keep is
+// exact and C is rounded once, so for operands of one scale the result is
+// closer to the exact product than 128 FP64 multiply-adds: relative error
+// 7e-17 against 3.8e-16 (256 x 256 x 128, N(0,1)), backward error of the whole
+// CALU 5.6e-15 against 1.2e-14 (n = 2048, N(0,1)).  What the digits keep is
 // relative to the largest magnitude of the row of A (column of B), so A's
 // columns are first brought to one scale and B's rows scaled back (powers of
-// two, column_exp_kernel): badly scaled rows of the matrix, which make the columns of L21 grow
-// from pivot to pivot while the rows of U12 shrink, then lose nothing.
+// two, column_exp_kernel), which undoes badly scaled rows of the matrix; and
+// an element that is still small beside its row's and column's largest is
+// found by tc_check_kernel and multiplied in FP64.
 // CALU + solve of n = 10240, b = 128: 681 -> 186 ms (622 ms of FP64 GEMM
 // became 120 ms here, most of it beside the next panel's tournament).
 // --------------------------------------------------------------------------
@@ -959,7 +1197,9 @@ __global__ void __launch_bounds__(256) column_exp_kernel(int m, const double *__
   }
 }
 
-size_t tc_f64_ws_bytes(int m, int n, int k) { return align256((size_t)k * 4) + 256 + tc_gemm_ws_bytes(m, n, k, kTcF64Slices); }
+size_t tc_f64_ws_bytes(int m, int n, int k) {
+  return align256((size_t)k * 4) + 256 + tc_gemm_ws_bytes_batched(m, n, k, kTcF64Slices, 1, true);
+}
 
 // One 128 x 64 tile of digits costs about 15 us however little of it is used
 // (three launches, 28 products); the FP64 kernel as much at 64 x 64 x 64.
@@ -972,7 +1212,7 @@ cudaError_t gemm_minus_f64_tc(int m, int n, int k, const double *A, int lda, con
   char *p = (char *)(((uintptr_t)ws + 255) & ~(uintptr_t)255);
   int *kexp = (int *)p;
   TcGemm g = schur_gemm(m, n, k, A, lda, B, ldb, C, ldc, kTcF64Slices, 1, skip);
-  g.full = 1;
+  g.keep = 2.5f / 8.0f;
   g.kexp = kexp;
   g.reuse_a = !first;
   if (first) {

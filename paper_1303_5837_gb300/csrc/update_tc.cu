@@ -70,19 +70,26 @@ __global__ void leaf_items_kernel(int nleaves, int L, int mk, int bk, int *top, 
   c[j] = rows < bk ? rows : bk;
 }
 
-size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, int S) {
+size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, int S, bool keep) {
   const int ch = nleaves < kChunkLeaves ? nleaves : kChunkLeaves;
   const size_t w = (size_t)ch * bk * ncols * 8;
-  size_t g = tc_gemm_ws_bytes_batched(bk, ncols, kHalfK, S, ch);           // W = Y^T C (per half)
-  g = g > tc_gemm_ws_bytes_batched(leaf_rows, ncols, bk, S, ch) ? g
-                                                                   : tc_gemm_ws_bytes_batched(leaf_rows, ncols, bk, S, ch);
+  const size_t g1 = tc_gemm_ws_bytes_batched(bk, ncols, kHalfK, S, ch, keep);  // W = Y^T C (per half)
+  const size_t g3 = tc_gemm_ws_bytes_batched(leaf_rows, ncols, bk, S, ch, keep);
+  const size_t g = g1 > g3 ? g1 : g3;
   const size_t items = 3 * align256((size_t)(nleaves + 1) * 4 * 8);
   (void)mk;
   return 2 * align256(w) + align256(g) + items + 256;
 }
 
-// The FP64 tree update from 7 digits: like the Schur update (gemm_tc.cu) its
-// products are exact and its error below that of FP64 multiply-adds.  It is a
+// The FP64 tree update from 7 digits.  As in the Schur update (gemm_tc.cu) an
+// element that is small beside its vectors' largest is multiplied in FP64, so
+// that heavy rows do not take the light ones' digits.  The line (kTreeKeep) is
+// a tenth of the Schur update's: sums of one or two terms (the top rows of a
+// leaf, the first reflectors of a merge) come near any line by chance, and at
+// 2.5 / 8 nearly every block that holds one would run in FP64.  An element's
+// error bound is therefore up to ten times that of FP64 multiply-adds; the
+// measured error of CAQR is 0.8 to 1.5 times that of the FP64 kernels (2000 x
+// 1400, the first rows weighted by 2^0 .. 2^40).  The update is a
 // chain of many small launches (three per contraction of up to 128 rows), so
 // it pays where the FP64 kernels would take longer than about 5 us per launch
 // at the 0.5 TFLOP/s they reach on the shapes near the line (1.07 wide, 0.2
@@ -98,7 +105,7 @@ bool tree_tc_pays(int mk, int bk, int ncols, int leaf_rows, const Plan &plan) {
 
 cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, int leaf_rows, const Plan &plan,
                              const double *Tp, double *C, int ldc, int ncols, const QrPanelWs &ws, void *tcws,
-                             int S, int exact, int *status, cudaStream_t st, int full) {
+                             int S, int exact, int *status, cudaStream_t st, float keep) {
   if (ncols <= 0) return cudaSuccess;
   const int L = leaf_rows, nl = plan.nleaves;
   const int ch = nl < kChunkLeaves ? nl : kChunkLeaves;  // a round of merges has fewer nodes
@@ -107,8 +114,8 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
   p += align256((size_t)ch * bk * ncols * 8);
   double *Wp = (double *)p;
   p += align256((size_t)ch * bk * ncols * 8);
-  size_t g = tc_gemm_ws_bytes_batched(bk, ncols, kHalfK, S, ch);
-  const size_t g3 = tc_gemm_ws_bytes_batched(L, ncols, bk, S, ch);
+  size_t g = tc_gemm_ws_bytes_batched(bk, ncols, kHalfK, S, ch, keep > 0.0f);
+  const size_t g3 = tc_gemm_ws_bytes_batched(L, ncols, bk, S, ch, keep > 0.0f);
   if (g3 > g) g = g3;
   void *gws = p;
   p += align256(g);
@@ -133,8 +140,12 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
     const int kk_last = L_last < bk ? L_last : bk;
     if ((e = cudaMemsetAsync(W, 0, wbytes, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(Wp, 0, wbytes, st)) != cudaSuccess) return e;
-    // W = Y^T C, in contraction halves of 128 leaf rows
-    for (int h = 0; h * kHalfK < L; ++h) {
+    // W = Y^T C, in contraction halves of 128 leaf rows; with keep the leaf's
+    // top last: there a column of Y is its unit diagonal and little else, and
+    // W already holds what the rows below gave
+    const int nh = (L + kHalfK - 1) / kHalfK;
+    for (int i = 0; i < nh; ++i) {
+      const int h = keep > 0.0f ? nh - 1 - i : i;
       TcGemm g1 = {};
       g1.A.X = P + (size_t)j0 * L + h * kHalfK;
       g1.A.sv = lda;
@@ -162,7 +173,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
       g1.sign = -1.0;
       g1.S = S;
       g1.exact = exact;
-      g1.full = full;
+      g1.keep = keep;
       if ((e = gemm_tc(g1, gws, status, st)) != cudaSuccess) return e;
     }
     // W' = T^T W
@@ -171,6 +182,8 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
     g2.A.sv = b;
     g2.A.sk = 1;
     g2.A.sb = (long long)b * b;
+    g2.A.shape = 2;  // T is upper triangular
+    g2.A.trans = 1;
     g2.A.nv = kk;
     g2.A.nv_last = kk_last;
     g2.A.K = kk;
@@ -189,7 +202,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
     g2.sign = -1.0;
     g2.S = S;
     g2.exact = exact;
-    g2.full = full;
+    g2.keep = keep;
     if ((e = gemm_tc(g2, gws, status, st)) != cudaSuccess) return e;
     // C -= Y W'
     TcGemm g3 = {};
@@ -211,7 +224,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
     g3.sign = 1.0;
     g3.S = S;
     g3.exact = exact;
-    g3.full = full;
+    g3.keep = keep;
     if ((e = gemm_tc(g3, gws, status, st)) != cudaSuccess) return e;
   }
 
@@ -265,7 +278,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
         g1.sign = -1.0;
         g1.S = S;
         g1.exact = exact;
-        g1.full = full;
+        g1.keep = keep;
         if ((e = gemm_tc(g1, gws, status, st)) != cudaSuccess) return e;
       }
       TcGemm g2 = {};
@@ -273,6 +286,8 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
       g2.A.sv = b;
       g2.A.sk = 1;
       g2.A.sb = (long long)b * b;
+      g2.A.shape = 2;  // T is upper triangular
+      g2.A.trans = 1;
       g2.A.nv = g2.A.nv_last = bk;
       g2.A.K = g2.A.K_last = bk;
       g2.B.X = W;
@@ -288,7 +303,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
       g2.sign = -1.0;
       g2.S = S;
       g2.exact = exact;
-      g2.full = full;
+      g2.keep = keep;
       if ((e = gemm_tc(g2, gws, status, st)) != cudaSuccess) return e;
       {
         ProfScope ps(kClsTreeApply, st, 0.0);
@@ -315,7 +330,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
         g3.sign = 1.0;
         g3.S = S;
         g3.exact = exact;
-        g3.full = full;
+        g3.keep = keep;
         if ((e = gemm_tc(g3, gws, status, st)) != cudaSuccess) return e;
       }
     }
