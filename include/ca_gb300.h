@@ -42,9 +42,10 @@
  *     two events per (device, caller stream) on first use (up to 64 pairs,
  *     beyond that plain stream order) and keeps them until the process exits.
  *     Every piece of work is ordered by events that start from and end on
- *     `stream`, so the caller sees ordinary stream semantics; results are
- *     bit-identical to the serial order.  Calls on one caller stream must not
- *     be enqueued from two host threads at once.
+ *     `stream`, so the caller sees ordinary stream semantics.  CALU's results
+ *     are bit-identical to the serial order; CAQR's agree to rounding (an FP64
+ *     update of few columns may add in another order than one of many).  Calls
+ *     on one caller stream must not be enqueued from two host threads at once.
  */
 #ifndef CA_GB300_H
 #define CA_GB300_H
