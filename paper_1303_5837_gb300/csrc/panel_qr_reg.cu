@@ -551,6 +551,10 @@ __global__ void __launch_bounds__(kRegThreads, 1) tsqr_creg_kernel(TsqrNodeArgs 
       }
       for (int qc = nd.rg + kCW; qc < b; qc += 16) Tg[i + (size_t)qc * b] = 0.0;  // a last panel narrower than b
     }
+    constexpr int kTRows = 16 * kCG;  // one row of T per half-warp of the cluster
+    if (rank == 0 && b > kTRows)      // b > 128 with at most 128 columns in the matrix: the rows past them
+      for (size_t idx = tid; idx < (size_t)(b - kTRows) * b; idx += kRegThreads)
+        Tg[kTRows + idx % (b - kTRows) + idx / (b - kTRows) * b] = 0.0;
   }
 #pragma unroll
   for (int s = 0; s < TS; ++s) {

@@ -210,3 +210,22 @@ def test_solve_does_not_read_what_an_earlier_one_left(ca, n, nrhs):
     ca.calu_getrs(F, ipiv, Y)
     torch.cuda.synchronize()
     assert np.abs(to_host(Y) - X).max() <= 1e-11
+
+
+@pytest.mark.parametrize("m,n,b,L,lv", [(600, 100, 200, 256, [(0, 0)]), (700, 128, 129, 700, [(0, 0)]),
+                                        (900, 64, 300, 300, [(0, 1)]), (100, 20, 150, 150, [(0, 0)])])
+def test_t_blocks_wider_than_the_matrix(ca, m, n, b, L, lv):
+    """A panel width beyond the matrix and beyond 128: every b x b block of the
+    store is written, zero outside the corner of the panel's T."""
+    A = inputs.gaussian(m, n, m + b)
+    t_o = oracle.make_tree(L, lv)
+    QR_o, T_o = oracle.caqr(A, b, t_o)
+    Ad = to_dev(A)
+    qtree = torch.full((ca.ca_caqr_workspace(m, n, b, ca.make_tree(L, lv))[0] // 8,), float("nan"), dtype=torch.float64,
+                       device="cuda")
+    ca.caqr_factor(Ad, b, ca.make_tree(L, lv), qtree=qtree)
+    torch.cuda.synchronize()
+    check(qr_err(to_host(Ad), QR_o, b), TOL, (m, n, b))
+    check(qtree_err(qtree.cpu().numpy(), T_o, QR_o, b, t_o, oracle.tree_counts), TOL, (m, n, b))
+    blocks = qtree.view(-1, b, b)
+    assert not torch.any(blocks[:, n:, :]) and not torch.any(blocks[:, :, n:])
