@@ -286,6 +286,12 @@ int ca_solve_status(const void *work, int *timed_out, cudaStream_t stream);
  * of the library, not thread-safe against solves being enqueued. */
 void ca_test_solve_hook(long long wait_cycles, int withhold);
 
+/* ca_test_cluster_hook: a test hook with no counterpart in the paper.
+ * Tournament nodes enqueued after this call use clusters of at most max_ctas
+ * CTAs wherever 8 hold their rows, as on a device that cannot place clusters
+ * beyond the portable size; <= 0 restores the default.  Host state, as above. */
+void ca_test_cluster_hook(int max_ctas);
+
 /* ------------------------------------------------------------------------ */
 /* Reduced-precision trailing update on the tensor cores                    */
 /* ------------------------------------------------------------------------ */

@@ -359,6 +359,7 @@ struct SolveWs {
 size_t solve_ws_bytes(int n);
 void solve_ws_carve(void *w, int n, SolveWs &s);
 void solve_test_hook(long long wait_cycles, int withhold_blk);
+void tslu_test_max_cluster(int n);  // clusters of at most n CTAs where 8 hold the rows (<= 0: the default)
 cudaError_t getrs_swap(int n, int nrhs, const int *ipiv, double *B, int ldb, cudaStream_t st,
                        const int *skip = nullptr);
 cudaError_t trsm_left(bool lower, bool unit, int n, int nrhs, const double *T, int ldt, double *B, int ldb,

@@ -2,7 +2,7 @@
 // stacked candidate rows of a merge: Sec. 3.2) held in registers.
 //
 // A node's rows are split in contiguous chunks over the G CTAs of one cluster
-// (G = 1, 2, 4, 8).  TPR threads hold one row: thread `sub` of a row keeps the
+// (G = 1, 2, 4, 8, 16).  TPR threads hold one row: thread `sub` of a row keeps the
 // columns k TPR + sub, k < CPT, in registers.  Rows never move: every row
 // carries the position it would have after the interchanges made so far (the
 // rule "first maximum in the physically swapped order" needs it), and a row
@@ -451,24 +451,62 @@ __global__ void __launch_bounds__(lu_reg_rows<TPR, CPT>() * TPR, CPT == 16 && TP
   if (nd.rank == 0 && tid < 32) lu_root_swaps(a, sm.sel, sm.work);
 }
 
+constexpr int kKeepBytes = (128 * 129 > 256 * 65 ? 128 * 129 : 256 * 65) * 8;  // most dynamic shared memory (root)
+
+// Whether the current device can place a cluster of kMaxG CTAs of this kernel
+// (more than the portable 8, so it depends on the device and its partition),
+// asked once per device, for the largest shape it is launched with.
+template <int TPR, int CPT>
+bool big_cluster_fits() {
+  static std::atomic<unsigned long long> asked{0}, fits{0};
+  const cudaError_t e = once_per_device(asked, [] {
+    auto *fn = tslu_reg_kernel<TPR, CPT, true>;
+    cudaError_t r = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (r == cudaSuccess) r = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kKeepBytes);
+    int dev = 0, n = 0;
+    if (r == cudaSuccess) r = cudaGetDevice(&dev);
+    if (r == cudaSuccess) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(kMaxG);
+      cfg.blockDim = dim3(lu_reg_rows<TPR, CPT>() * TPR);
+      cfg.dynamicSmemBytes = kKeepBytes;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = kMaxG;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
+        cudaGetLastError();  // a refusal is an answer, not a failure of the call that asks
+        n = 0;
+      }
+      if (n > 0 && dev < kMaxDevices) fits.fetch_or(1ull << dev, std::memory_order_relaxed);
+    }
+    return r;
+  });
+  int dev = 0;
+  return e == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess && dev < kMaxDevices &&
+         (fits.load(std::memory_order_relaxed) >> dev & 1ull);
+}
+
+bool big_cluster_fits(int bk, int rloc) {  // of the kernel that launch_tslu_reg takes
+  if (bk <= 16) return big_cluster_fits<1, 16>();
+  if (bk <= 32) return big_cluster_fits<2, 16>();
+  if (bk <= 64) return rloc <= 64 ? big_cluster_fits<4, 16>() : big_cluster_fits<2, 32>();
+  return big_cluster_fits<4, 32>();
+}
+
 template <int TPR, int CPT, bool CL>
 cudaError_t launch_reg1(const TsluNodeArgs &a, int nodes, int G, cudaStream_t st) {
-  if (G > 8) {
-    static std::atomic<unsigned long long> big{0};
-    cudaError_t e = once_per_device(big, [] {
-      return cudaFuncSetAttribute(tslu_reg_kernel<TPR, CPT, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    });
-    if (e != cudaSuccess) return e;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nodes * G);
   cfg.blockDim = dim3((a.rloc * TPR + 31) / 32 * 32);
   cfg.stream = st;
   if (a.is_root) {
-    constexpr int kMost = (128 * 129 > 256 * 65 ? 128 * 129 : 256 * 65) * 8;
     static std::atomic<unsigned long long> init{0};
     cudaError_t e = once_per_device(init, [] {
-      return cudaFuncSetAttribute(tslu_reg_kernel<TPR, CPT, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+      return cudaFuncSetAttribute(tslu_reg_kernel<TPR, CPT, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKeepBytes);
     });
     if (e != cudaSuccess) return e;
     cfg.dynamicSmemBytes = (size_t)a.rloc * ((a.bk + TPR - 1) / TPR * TPR | 1) * 8;
@@ -490,21 +528,31 @@ cudaError_t launch_reg(const TsluNodeArgs &a, int nodes, int G, cudaStream_t st)
 
 }  // namespace
 
+static std::atomic<int> g_max_cluster{16};  // test hook
+
+void tslu_test_max_cluster(int n) { g_max_cluster.store(n > 0 ? n : 16); }
+
 // Cluster size of a node of R rows and bk columns (a round of `nodes`), and
 // the rows per CTA; 0 when the rows do not fit the registers of 8 CTAs.  The
 // smallest cluster that holds the rows, doubled while the round's CTAs still
 // find an SM each and a CTA keeps at least kMinRows rows (128 x 64: 125 us on
 // one CTA, 121 on 2, 104 on 4, 109 on 8; 256 x 64: 201, 150, 123, 109).
 // Sixteen CTAs (beyond the portable cluster size, so never needed to hold the
-// rows) for at most six nodes: 1024 x 128 471 -> 344 us, 512 x 128 317 -> 291.
+// rows, and only where the device can place such clusters) for rounds that
+// fill at most two thirds of the SMs (six nodes of 152): 1024 x 128
+// 471 -> 344 us, 512 x 128 317 -> 291.  The result does not depend on G.
 int tslu_reg_cluster(int R, int bk, int nodes, int *rloc) {
   if (bk < 1 || bk > 128 || R < 1) return 0;
   const int rmax = bk <= 64 ? 256 : 128;
   constexpr int kMinRows = 24;
-  int G = 1;
+  int sms = 0, G = 1;
+  if (device_sm_count(&sms) != cudaSuccess) return 0;
   while (G < 8 && (R + G - 1) / G > rmax) G *= 2;
   if ((R + G - 1) / G > rmax) return 0;
-  while (G < kMaxG && (G < 8 || nodes * 16 <= 96) && nodes * G * 2 <= 152 && (R + 2 * G - 1) / (2 * G) >= kMinRows) G *= 2;
+  while (G < 8 && (long long)nodes * G * 2 <= sms && (R + 2 * G - 1) / (2 * G) >= kMinRows) G *= 2;
+  if (G == 8 && (long long)nodes * kMaxG * 3 <= 2 * sms && (R + kMaxG - 1) / kMaxG >= kMinRows &&
+      g_max_cluster.load() >= kMaxG && big_cluster_fits(bk, (R + kMaxG - 1) / kMaxG))
+    G = kMaxG;
   *rloc = (R + G - 1) / G;
   return G;
 }
