@@ -91,17 +91,21 @@ size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, i
 // measured error of CAQR is 0.8 to 1.5 times that of the FP64 kernels (2000 x
 // 1400, the first rows weighted by 2^0 .. 2^40).  The update is a
 // chain of many small launches (split, check and product per contraction of up
-// to 128 rows), so it pays where the FP64 kernels would take longer than about
-// 8 us per launch at the 0.5 TFLOP/s they reach on the shapes near the line
-// (1.07 wide, 0.2 narrow).  CAQR in ms with the line at 5, 8, 12 us and without
-// digits: 1024 x 1024 (b = 64, 128-row leaves) 11.9, 12.1, 12.5, 12.3;
-// 3001 x 750 with its solve 22.6, 21.2, 21.4, 22.7; 2000 x 2000 (b = 64) 34.1,
-// 34.6, 35.1, 41.1; 6144 x 6144 (1024-row leaves) 145.8, 143.3, 138.8, 389.
+// to 128 rows), so it pays where the FP64 kernels would take longer than some
+// time per launch at the 0.5 TFLOP/s they reach on the shapes near the line
+// (1.07 wide, 0.2 narrow).  That time depends on the panel's width: below 64
+// columns half of a digit tile is padding, above 64 the FP64 kernels use their
+// lanes better.  CAQR in ms with the line at 3, 5, 8, 12, 20 us and without
+// digits: b = 32, 1500 x 1500: 30.8, 29.3, 28.3, 27.9, 27.8, 28.0;
+// b = 64 (128-row leaves), 1024 x 1024: 11.7, 11.9, 12.1, 12.5, 12.3, 12.3,
+// 2000 x 2000: 34.2, 34.1, 34.6, 35.1, 37.2, 41.1;
+// b = 128, 3001 x 750 with its solve: 23.1, 22.6, 21.2, 21.4, 22.0, 22.7,
+// 6144 x 6144 (1024-row leaves): 146.8, 145.8, 143.3, 138.8, 139.5, 389.
 bool tree_tc_pays(int mk, int bk, int ncols, int leaf_rows, const Plan &plan) {
   int launches = ((leaf_rows + kHalfK - 1) / kHalfK + 2) * 3 + 3;
   for (int r = 0; r < plan.nrounds; ++r) launches += 3 * (2 * plan.r[r].max_cnt - 1) + 4;
   const double fp64_us = 4.0 * mk * bk * (double)ncols / 0.5e6;
-  return bk >= 16 && bk <= 128 && fp64_us > 8.0 * launches;
+  return bk >= 16 && bk <= 128 && fp64_us > (bk < 64 ? 12.0 : bk == 64 ? 5.0 : 10.0) * launches;
 }
 
 cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, int leaf_rows, const Plan &plan,
