@@ -292,6 +292,15 @@ void ca_test_solve_hook(long long wait_cycles, int withhold);
  * beyond the portable size; <= 0 restores the default.  Host state, as above. */
 void ca_test_cluster_hook(int max_ctas);
 
+/* ca_test_panel_hook: a test hook with no counterpart in the paper.  With
+ * withhold = 1, the last CTA of every cluster of the register-resident panel
+ * nodes (TSLU, TSQR) enqueued after this call sends the others nothing, so
+ * the cluster's waits run out after wait_cycles SM clock
+ * cycles (<= 0: the default, about 2 s) and dev_info[1] gets
+ * CA_STATUS_PANEL_TIMEOUT; withhold = 0 restores normal nodes.  Host state,
+ * as above. */
+void ca_test_panel_hook(long long wait_cycles, int withhold);
+
 /* ------------------------------------------------------------------------ */
 /* Reduced-precision trailing update on the tensor cores                    */
 /* ------------------------------------------------------------------------ */

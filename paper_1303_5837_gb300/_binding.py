@@ -104,7 +104,7 @@ SYMBOLS = ("ca_strerror", "ca_calu_workspace", "ca_caqr_workspace", "ca_geqrs_wo
            "ca_gemm_mixed_workspace", "ca_gemm_minus_mixed", "ca_calu_mixed_workspace",
            "calu_factor_mixed", "ca_gesv_mixed_workspace", "calu_gesv_mixed", "ca_caqr_mixed_workspace",
            "caqr_factor_mixed", "ca_batched_plan", "ca_batched_factor", "ca_solve_status",
-           "ca_getrs_workspace", "ca_test_solve_hook", "ca_test_cluster_hook", "tslu_noalloc", "ca_peak_probe",
+           "ca_getrs_workspace", "ca_test_solve_hook", "ca_test_cluster_hook", "ca_test_panel_hook", "tslu_noalloc", "ca_peak_probe",
            "ca_gels_mixed_workspace", "caqr_gels_mixed")
 KERNEL_CLASSES = ("tslu_node", "laswp", "lu_finish", "trsm_u12", "gemm_fp64", "tsqr_node",
                   "tree_apply", "solve", "split_bf16", "gemm_tc", "refine", "batched",
@@ -142,6 +142,8 @@ def load(build_if_missing: bool = True):
     L.ca_test_solve_hook.restype = None
     L.ca_test_cluster_hook.argtypes = [I]
     L.ca_test_cluster_hook.restype = None
+    L.ca_test_panel_hook.argtypes = [ctypes.c_longlong, I]
+    L.ca_test_panel_hook.restype = None
     L.ca_peak_probe.argtypes = [I, I, I, P, P]
     L.ca_gels_mixed_workspace.argtypes = [I, I, I, I, T, I, I, PS, PS]
     L.caqr_gels_mixed.argtypes = [I, I, I, P, I, I, T, I, I, P, I, P, S, P, I, P, I, P, S, I, ctypes.c_double,
@@ -357,6 +359,12 @@ def ca_test_cluster_hook(max_ctas: int = 0):
     """Test hook: tournament nodes use clusters of at most max_ctas CTAs where 8
     hold their rows (0: the default)."""
     load().ca_test_cluster_hook(int(max_ctas))
+
+
+def ca_test_panel_hook(wait_cycles: int = 0, withhold: bool = False):
+    """Test hook: withhold=True keeps one CTA's rows from its cluster in the next
+    panel nodes, so their waits run out after wait_cycles."""
+    load().ca_test_panel_hook(int(wait_cycles), 1 if withhold else 0)
 
 
 # ---------------------------------------------------------------------------

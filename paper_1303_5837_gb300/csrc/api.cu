@@ -521,6 +521,8 @@ int ca_solve_status(const void *work, int *timed_out, cudaStream_t stream) {
   return CA_OK;
 }
 
+void ca_test_panel_hook(long long wait_cycles, int withhold) { panel_test_hook(wait_cycles, withhold); }
+
 void ca_test_cluster_hook(int max_ctas) { tslu_test_max_cluster(max_ctas); }
 
 void ca_test_solve_hook(long long wait_cycles, int withhold) { solve_test_hook(wait_cycles, withhold ? 0 : -1); }

@@ -265,6 +265,8 @@ struct TsqrNodeArgs {
   int rloc, ld;   // tile rows per CTA, tile leading dimension (odd)
   int *dev_info;
   int fixed;      // keep the order of sums and the library's square root (panel_qr_fixed.cu)
+  long long wait_limit;  // cluster nodes: SM clocks a wait may take
+  int withhold;          // test hook: the last CTA of a cluster sends nothing
 };
 // Register-resident TSQR nodes (panel_qr_reg.cu) for nodes of at most 256
 // rows and 64 columns held by one CTA; *done = false when the shape is not
@@ -359,6 +361,7 @@ struct SolveWs {
 size_t solve_ws_bytes(int n);
 void solve_ws_carve(void *w, int n, SolveWs &s);
 void solve_test_hook(long long wait_cycles, int withhold_blk);
+void panel_test_hook(long long wait_cycles, int withhold);  // cluster nodes (panel_lu_reg.cu, panel_qr_reg.cu)
 void tslu_test_max_cluster(int n);  // clusters of at most n CTAs where 8 hold the rows (<= 0: the default)
 cudaError_t getrs_swap(int n, int nrhs, const int *ipiv, double *B, int ldb, cudaStream_t st,
                        const int *skip = nullptr);

@@ -24,6 +24,8 @@ struct TsluNodeArgs {
   int ipiv_base;    // kb
   const int *skip;  // nonzero: a stage enqueued ahead that is not needed, do nothing
   int *dev_info;    // [0] info, [1] status
+  long long wait_limit;  // register nodes: SM clocks a wait may take
+  int withhold;          // test hook: the last CTA of a cluster sends nothing
 };
 
 // register-resident nodes (panel_lu_reg.cu)

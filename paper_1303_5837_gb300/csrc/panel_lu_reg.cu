@@ -42,6 +42,7 @@
 #include <climits>
 
 #include "ca_internal.cuh"
+#include "cluster_copy.cuh"
 #include "device_once.cuh"
 #include "fp64_int.cuh"
 #include "lu_node.cuh"
@@ -59,8 +60,6 @@ struct alignas(16) Key {
 constexpr int kMaxG = 16;
 constexpr int kMaxWarps = 16;
 
-constexpr long long kLuWait = 4000000000ll;  // about 2 s of SM clock
-
 template <int TPR, int CPT, bool CL>
 struct alignas(16) LuRegSmem {
   // a published row: its Key, 1 / pivot, a pad, then the threads' parts four
@@ -70,6 +69,7 @@ struct alignas(16) LuRegSmem {
   double stage[CL ? 2 : 1][kRow];      // cluster: the CTA's row on its way out, by column parity
   Key keys[2][kMaxWarps];              // best of every warp of this CTA, by column parity
   unsigned long long bar[3];                  // cluster: the rows of a column have arrived
+  int gave_up;                                // a CTA of the cluster gave up waiting
   int sel[128];                               // root, rank 0: labels of the chosen rows in pivot order
   int work[3 * 128];
 };
@@ -82,40 +82,6 @@ __device__ __forceinline__ void cl_arrive() {
 __device__ __forceinline__ void cl_wait() {
   __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-// bytes of this CTA's shared memory to CTA `rank`'s, counted on its barrier
-__device__ __forceinline__ void bulk_to(const void *dst, const void *src, unsigned bytes, const void *bar, int rank) {
-  asm volatile(
-      "{\n\t.reg .b32 d, m;\n\t"
-      "mapa.shared::cluster.u32 d, %0, %4;\n\t"
-      "mapa.shared::cluster.u32 m, %2, %4;\n\t"
-      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [d], [%1], %3, [m];\n\t}\n" ::"r"(
-          smem_addr(dst)),
-      "r"(smem_addr(src)), "r"(smem_addr(bar)), "r"(bytes), "r"(rank)
-      : "memory");
-}
-__device__ __forceinline__ void bar_expect(unsigned long long *bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-// false when the phase did not complete within the limit
-__device__ __forceinline__ bool bar_wait(unsigned long long *bar, unsigned parity) {
-  const unsigned addr = smem_addr(bar);
-  const long long t0 = clock64();
-  while (true) {
-    unsigned done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (clock64() - t0 > kLuWait) return false;
-  }
 }
 
 // Largest key of the warp, smallest position among equal keys (on every lane).
@@ -141,6 +107,8 @@ struct Node {
   int pos;  // position of the row after the interchanges so far; -1: no row
   bool dead = false;  // cluster: a wait gave up; nothing is waited for any more
   int *status;
+  long long limit;
+  int nsend;          // CTAs this one sends its rows to: G, or 0 after a give-up (test hook: always)
 
   __device__ __forceinline__ explicit Node(LuRegSmem<TPR, CPT, CL> &s) : cl(cg::this_cluster()), sm(s) {}
 
@@ -197,7 +165,7 @@ struct Node {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copies read what was just written
       __syncwarp();
       const int b3 = j % 3;
-      if (lane < G) bulk_to(sm.u[b3 * kMaxG + rank], u, row_bytes(nb), &sm.bar[b3], lane);
+      if (lane < nsend) bulk_to(sm.u[b3 * kMaxG + rank], u, row_bytes(nb), &sm.bar[b3], lane);
     }
   }
 
@@ -205,11 +173,12 @@ struct Node {
   __device__ __forceinline__ const double *receive(int j, unsigned long long &key, int &p) {
     if constexpr (CL) {
       const int b3 = j % 3;
-      if (!dead && !bar_wait(&sm.bar[b3], (j / 3) & 1)) {
+      if (!dead && !bar_wait(&sm.bar[b3], (j / 3) & 1, limit)) {
         dead = true;
-        if (lane == 0 && status) atomicOr(status, CA_STATUS_PANEL_TIMEOUT);
+        nsend = 0;
+        tell_gave_up(&sm.gave_up, status);
       }
-      if (warp == 0 && lane == 0) expect(j + 3);
+      if (threadIdx.x == 0 && !dead) expect(j + 3);
       unsigned long long mk = 0;
       int mp = INT_MAX;
       if (lane < G) {
@@ -411,12 +380,15 @@ __global__ void __launch_bounds__(lu_reg_rows<TPR, CPT>() * TPR, CPT == 16 && TP
 
   // ---- column 0's pivot row, then every column ----------------------------
   nd.status = a.dev_info ? a.dev_info + 1 : nullptr;
+  nd.limit = a.wait_limit;
+  nd.nsend = a.withhold && nd.rank == nd.G - 1 ? 0 : nd.G;
   if constexpr (CL) {
     if (tid == 0) {
       for (int q = 0; q < 3; ++q)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sm.bar[q])) : "memory");
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       for (int q = 0; q < 3; ++q) nd.expect(q);
+      sm.gave_up = 0;
     }
     cl_arrive();  // the barriers of every CTA are set up before anything is sent to them
     cl_wait();
@@ -429,25 +401,30 @@ __global__ void __launch_bounds__(lu_reg_rows<TPR, CPT>() * TPR, CPT == 16 && TP
   run.keep = a.is_root && lab >= 0 ? keep + (size_t)row * ldk + nd.sub : nullptr;
   nd.columns(run);
 
-  // ---- outputs: labels in pivot order -------------------------------------
-  const bool chosen = nd.pos >= 0 && nd.pos < nd.kmax;
-  if (chosen && nd.sub == 0) a.cand_out[(size_t)node * a.cand_ld + nd.pos] = lab;
-  if (nd.rank == 0 && tid == 0) a.ncand_out[node] = nd.kmax;
-  if (!a.is_root) {
-    if constexpr (CL) {  // nothing is on its way to a CTA that has left
+  // ---- outputs: labels in pivot order; root: L11 \ U11 of the chosen rows ---
+  auto outputs = [&] {
+    const bool chosen = nd.pos >= 0 && nd.pos < nd.kmax;
+    if (chosen && nd.sub == 0) a.cand_out[(size_t)node * a.cand_ld + nd.pos] = lab;
+    if (nd.rank == 0 && tid == 0) a.ncand_out[node] = nd.kmax;
+    if (!a.is_root || !chosen) return;
+    for (int col = nd.sub; col < bk; col += TPR) a.lu11[nd.pos + (size_t)col * a.cand_ld] = keep[(size_t)row * ldk + col];
+    if (nd.sub == 0) *nd.cl.map_shared_rank(&sm.sel[nd.pos], 0) = lab;
+  };
+  outputs();
+  if (CL || a.is_root) {  // nothing is on its way to a CTA that has left; rank 0 holds every chosen label
+    cl_arrive();
+    cl_wait();
+  }
+  if constexpr (CL)
+    if (cluster_gave_up(&sm.gave_up)) {
+      // positions may be anything: the node's first rows stand in for the
+      // choice (valid labels, each once; the status tells)
+      nd.pos = lab >= 0 ? p : -1;
+      outputs();
       cl_arrive();
       cl_wait();
     }
-    return;
-  }
-
-  // root: L11 \ U11 of the chosen rows, and the row permutation
-  if (chosen) {
-    for (int col = nd.sub; col < bk; col += TPR) a.lu11[nd.pos + (size_t)col * a.cand_ld] = keep[(size_t)row * ldk + col];
-    if (nd.sub == 0) *nd.cl.map_shared_rank(&sm.sel[nd.pos], 0) = lab;
-  }
-  cl_arrive();
-  cl_wait();  // rank 0 holds every chosen label; nothing is on its way to a CTA that has left
+  if (!a.is_root) return;
   if (nd.rank == 0 && tid < 32) lu_root_swaps(a, sm.sel, sm.work);
 }
 
@@ -518,7 +495,10 @@ cudaError_t launch_reg1(const TsluNodeArgs &a, int nodes, int G, cudaStream_t st
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tslu_reg_kernel<TPR, CPT, CL>, a);
+  TsluNodeArgs args = a;
+  args.wait_limit = panel_wait_limit();
+  args.withhold = panel_withhold();
+  return cudaLaunchKernelEx(&cfg, tslu_reg_kernel<TPR, CPT, CL>, args);
 }
 
 template <int TPR, int CPT>

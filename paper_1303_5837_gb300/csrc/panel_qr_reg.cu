@@ -25,6 +25,7 @@
 // balanced, where a shared-memory tile with column-per-thread dot products
 // leaves half the warps idle once fewer than half the columns remain.
 #include "ca_internal.cuh"
+#include "cluster_copy.cuh"
 #include "device_once.cuh"
 #include "qr_node_reg.cuh"
 
@@ -195,7 +196,6 @@ cudaError_t launch_reg(const TsqrNodeArgs &a, int nodes, cudaStream_t st) {
 // front of the copies) and had received this CTA's column j - 1.
 // ---------------------------------------------------------------------------
 constexpr int kCG = 8;    // CTAs per node
-constexpr long long kQrWait = 4000000000ll;  // about 2 s of SM clock
 
 template <int TC, int TS>
 struct alignas(16) CRegSmem {
@@ -209,38 +209,8 @@ struct alignas(16) CRegSmem {
   double tau[kCW], scal[kCW];
   double beta;
   unsigned long long bar[2];   // column parity: sums and row have arrived
+  int gave_up;                 // a CTA of the cluster gave up waiting
 };
-
-__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bulk_to(const void *dst, const void *src, unsigned bytes, const void *bar, int rank) {
-  asm volatile(
-      "{\n\t.reg .b32 d, m;\n\t"
-      "mapa.shared::cluster.u32 d, %0, %4;\n\t"
-      "mapa.shared::cluster.u32 m, %2, %4;\n\t"
-      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [d], [%1], %3, [m];\n\t}\n" ::"r"(
-          smem_addr(dst)),
-      "r"(smem_addr(src)), "r"(smem_addr(bar)), "r"(bytes), "r"(rank)
-      : "memory");
-}
-__device__ __forceinline__ void bar_expect(unsigned long long *bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool bar_wait(unsigned long long *bar, unsigned parity) {
-  const unsigned addr = smem_addr(bar);
-  const long long t0 = clock64();
-  while (true) {
-    unsigned done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (clock64() - t0 > kQrWait) return false;
-  }
-}
 
 // What the column steps of one thread share.
 template <int TC, int TS>
@@ -254,6 +224,8 @@ struct CNode {
   double T[kCTC];                     // row 8 hw + rank of T, columns rg + 16 t
   bool dead;                          // a wait gave up; nothing is waited for any more
   int *status;
+  long long limit;
+  int nsend;                          // CTAs this one sends to: 8, or 0 after a give-up (test hook: always)
 
   __device__ __forceinline__ explicit CNode(CRegSmem<TC, TS> &s) : sm(s) {}
   __device__ __forceinline__ int node_row(int s) const {
@@ -324,18 +296,19 @@ struct CNode {
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copies read what was just written
       __syncthreads();
-      if (threadIdx.x < kCG) {
+      if ((int)threadIdx.x < nsend) {
         const unsigned bytes = 8u * bkw;
         bulk_to(sm.in[q][rank], sm.out[q], bytes, &sm.bar[q], threadIdx.x);
         if ((cyc ? j % kCG : j / (16 * TS)) == rank) bulk_to(sm.row[q], sm.out[q] + kCW, bytes, &sm.bar[q], threadIdx.x);
       }
       if (j > 0) t_column(j - 1);
-      if (!dead && !bar_wait(&sm.bar[q], (j >> 1) & 1)) {
+      if (!dead && !bar_wait(&sm.bar[q], (j >> 1) & 1, limit)) {
         dead = true;
-        if ((threadIdx.x & 31) == 0 && status) atomicOr(status, CA_STATUS_PANEL_TIMEOUT);
+        nsend = 0;
+        tell_gave_up(&sm.gave_up, status);
       }
       if (threadIdx.x < kCW) {  // one warp per SM sub-partition adds the partials
-        if (threadIdx.x == 0 && j + 2 < kmax) bar_expect(&sm.bar[q], 8u * bkw * (kCG + 1));
+        if (threadIdx.x == 0 && j + 2 < kmax && !dead) bar_expect(&sm.bar[q], 8u * bkw * (kCG + 1));
         double v = sm.in[q][0][threadIdx.x];
 #pragma unroll
         for (int r = 1; r < kCG; ++r) v += sm.in[q][r][threadIdx.x];
@@ -452,6 +425,8 @@ __global__ void __launch_bounds__(kRegThreads, 1) tsqr_creg_kernel(TsqrNodeArgs 
   nd.c0 = nd.nk = nd.h = 0;
   nd.dead = false;
   nd.status = a.dev_info ? a.dev_info + 1 : nullptr;
+  nd.limit = a.wait_limit;
+  nd.nsend = a.withhold && rank == kCG - 1 ? 0 : kCG;
   if (!a.is_leaf) {
     const int c0 = a.c_in[start], h = a.c_in[start + 1];
     bool same = true;
@@ -521,12 +496,14 @@ __global__ void __launch_bounds__(kRegThreads, 1) tsqr_creg_kernel(TsqrNodeArgs 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     for (int q = 0; q < 2; ++q)
       if (q < nd.kmax) bar_expect(&sm.bar[q], 8u * nd.bkw * (kCG + 1));
+    sm.gave_up = 0;
   }
   // the zeros above come before the copies into the same buffers
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   cl.sync();  // every CTA's barriers are set up before anything is sent to them
   nd.template blocks<0>();
   cl.sync();  // nothing is on its way to a CTA that has left; tau, scal and z are final
+  if (cluster_gave_up(&sm.gave_up)) cl.sync();
   if (nd.kmax > 0) nd.t_column(nd.kmax - 1);
 
   // v = s x below the diagonal of every reflector column
@@ -585,7 +562,10 @@ cudaError_t launch_creg(const TsqrNodeArgs &a, int nodes, cudaStream_t st) {
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tsqr_creg_kernel<TC, TS>, a);
+  TsqrNodeArgs args = a;
+  args.wait_limit = panel_wait_limit();
+  args.withhold = panel_withhold();
+  return cudaLaunchKernelEx(&cfg, tsqr_creg_kernel<TC, TS>, args);
 }
 
 }  // namespace
@@ -624,6 +604,17 @@ cudaError_t launch_tsqr_reg(const TsqrNodeArgs &a, int nodes, int rows, cudaStre
   }
   if (rows <= 128) return launch_reg<4, 8>(a, nodes, st);
   return launch_reg<4, 16>(a, nodes, st);
+}
+
+// Test hook of the cluster nodes here and in panel_lu_reg.cu.
+static std::atomic<long long> g_panel_wait{kPanelWait};
+static std::atomic<int> g_panel_withhold{0};
+
+long long panel_wait_limit() { return g_panel_wait.load(); }
+int panel_withhold() { return g_panel_withhold.load(); }
+void panel_test_hook(long long wait_cycles, int withhold) {
+  g_panel_wait.store(wait_cycles > 0 ? wait_cycles : kPanelWait);
+  g_panel_withhold.store(withhold);
 }
 
 }  // namespace cagb
