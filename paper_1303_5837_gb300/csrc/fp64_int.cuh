@@ -17,7 +17,7 @@ __device__ __forceinline__ bool int_range(double v) {
   return E - 64u < 0x7ffu - 128u;
 }
 
-// 2^62 / m, m = |v| / 2^(E - 1023) in [1, 2): at most 16 units off (truncations
+// 2^63 / m, m = |v| / 2^(E - 1023) in [1, 2): at most 16 units off (truncations
 // of 1, 4 and 8 units, e^3 below 1).
 __device__ __forceinline__ unsigned long long recip_q62(unsigned long long M) {
   float x;
@@ -37,7 +37,7 @@ __device__ __forceinline__ double recip_near(double v) {
   return __longlong_as_double((long long)(((bits >> 63) << 63) | (((unsigned long long)(2044 - E) << 52) + mant)));
 }
 
-// The correctly rounded 1 / v, or 0 where the last ten bits of 2^62 / m lie
+// The correctly rounded 1 / v, or 0 where the last ten bits of 2^63 / m lie
 // within 24 of a tie (1 in 20) or v is outside int_range.
 __device__ __forceinline__ double recip_exact_or_zero(double v) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(v);

@@ -580,6 +580,10 @@ constexpr int kCregNodes = 38;
 
 bool tsqr_creg_fits(int rows, int bk, int nodes) {
   if (bk < 1 || bk > 128 || rows < 1 || rows > 128 * kCG) return false;
+  // (the shared-memory node sums x / (alpha - beta), this one x as it is, whose
+  // products with a much smaller column may underflow: shapes that always had
+  // the former keep it)
+  if (bk > 64 && rows <= 128) return false;
   return !tsqr_reg_fits(rows, bk) || nodes <= kCregNodes;
 }
 

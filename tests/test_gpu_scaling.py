@@ -45,6 +45,24 @@ def test_batched_qr_of_small_columns(ca, name, first, rest, m, n, L):
     assert np.all(np.abs(got - want) <= (m + 10) * np.finfo(dt).eps * np.linalg.norm(C, axis=0))
 
 
+@pytest.mark.parametrize("m,n,L", [(100, 100, 100), (128, 70, 128), (120, 120, 128)])
+def test_tsqr_of_small_columns(ca, m, n, L):
+    """The same in a single node of more than 64 columns and up to 128 rows."""
+    A = inputs.gaussian(m, n, m + n)
+    C = A[:, 1:].copy()
+    a = A[:, 0].copy()
+    A[:, 0] *= 1e-150
+    A[:, 1:] *= 1e-170
+    dev = to_dev(A)
+    ca.tsqr(dev, ca.make_tree(L))
+    beta = -np.copysign(np.linalg.norm(a), a[0])
+    v = a.copy()
+    v[0] -= beta
+    want = C[0] - v[0] * (2.0 / (v @ v)) * (v @ C)
+    got = dev[0, 1:].cpu().numpy() / 1e-170
+    assert np.all(np.abs(got - want) <= (m + 12) * 2.0 ** -52 * np.linalg.norm(C, axis=0))
+
+
 def to_dev(A):
     return torch.from_numpy(np.ascontiguousarray(np.asarray(A).T)).cuda().t()
 
