@@ -45,24 +45,24 @@ __device__ __forceinline__ bool bar_try(unsigned addr, unsigned parity) {  // wa
       : "memory");
   return done != 0;
 }
-static __device__ __noinline__ bool bar_wait_slow(unsigned addr, unsigned parity, long long limit) {
-  const long long t0 = clock64();
-  while (!bar_try(addr, parity))
-    if (clock64() - t0 > limit) return false;
-  return true;
-}
 // false when the phase did not complete within the limit
 __device__ __forceinline__ bool bar_wait(unsigned long long *bar, unsigned parity, long long limit) {
   const unsigned addr = smem_addr(bar);
-  return bar_try(addr, parity) || bar_wait_slow(addr, parity, limit);
+  const long long t0 = clock64();
+  while (true) {
+    if (bar_try(addr, parity)) return true;
+    if (clock64() - t0 > limit) return false;
+  }
 }
 
-// A thread that gave up tells every CTA of the cluster (flag: a word of shared
-// memory, zero before the first exchange) and, once a warp, the host.
-static __device__ __noinline__ void tell_gave_up(int *flag, int *status) {
-  cg::cluster_group cl = cg::this_cluster();
-  for (int r = 0; r < (int)cl.num_blocks(); ++r) atomicExch(cl.map_shared_rank(flag, r), 1);
-  if ((threadIdx.x & 31) == 0 && status) atomicOr(status, CA_STATUS_PANEL_TIMEOUT);
+// After the last column: if a thread of this CTA gave up, every CTA of the
+// cluster is told (flag: a word of shared memory, zero before the first
+// exchange), and the host.  Every thread calls it, outside the column loops;
+// inline, because a call costs the 254-register TSQR node 2 % of its time.
+__device__ __forceinline__ void tell_gave_up(cg::cluster_group &cl, bool dead, int *flag, int *status) {
+  if (!__syncthreads_or(dead)) return;
+  for (int r = threadIdx.x; r < (int)cl.num_blocks(); r += blockDim.x) atomicExch(cl.map_shared_rank(flag, r), 1);
+  if (dead && status) atomicOr(status, CA_STATUS_PANEL_TIMEOUT);
 }
 
 // After the cluster barrier that follows the last exchange: whether any thread

@@ -176,7 +176,6 @@ struct Node {
       if (!dead && !bar_wait(&sm.bar[b3], (j / 3) & 1, limit)) {
         dead = true;
         nsend = 0;
-        tell_gave_up(&sm.gave_up, status);
       }
       if (threadIdx.x == 0 && !dead) expect(j + 3);
       unsigned long long mk = 0;
@@ -411,6 +410,7 @@ __global__ void __launch_bounds__(lu_reg_rows<TPR, CPT>() * TPR, CPT == 16 && TP
     if (nd.sub == 0) *nd.cl.map_shared_rank(&sm.sel[nd.pos], 0) = lab;
   };
   outputs();
+  if constexpr (CL) tell_gave_up(nd.cl, nd.dead, &sm.gave_up, nd.status);
   if (CL || a.is_root) {  // nothing is on its way to a CTA that has left; rank 0 holds every chosen label
     cl_arrive();
     cl_wait();

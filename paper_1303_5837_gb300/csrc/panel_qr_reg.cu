@@ -305,7 +305,6 @@ struct CNode {
       if (!dead && !bar_wait(&sm.bar[q], (j >> 1) & 1, limit)) {
         dead = true;
         nsend = 0;
-        tell_gave_up(&sm.gave_up, status);
       }
       if (threadIdx.x < kCW) {  // one warp per SM sub-partition adds the partials
         if (threadIdx.x == 0 && j + 2 < kmax && !dead) bar_expect(&sm.bar[q], 8u * bkw * (kCG + 1));
@@ -502,6 +501,7 @@ __global__ void __launch_bounds__(kRegThreads, 1) tsqr_creg_kernel(TsqrNodeArgs 
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   cl.sync();  // every CTA's barriers are set up before anything is sent to them
   nd.template blocks<0>();
+  tell_gave_up(cl, nd.dead, &sm.gave_up, nd.status);
   cl.sync();  // nothing is on its way to a CTA that has left; tau, scal and z are final
   if (cluster_gave_up(&sm.gave_up)) cl.sync();
   if (nd.kmax > 0) nd.t_column(nd.kmax - 1);
