@@ -146,3 +146,22 @@ def test_all_cores_oracle_baseline():
     d = bench.cpu_baseline_all_cores(a, cores=2)
     assert d is not None and d["cores"] == 2 and d["kind"] == "oracle"
     assert d["value"] > 0 and d["seconds"] > 0 and "2 concurrent copies" in d["sample"]
+
+
+def test_headline_line_is_short_and_complete():
+    """Standard output carries the contract's keys in a line of a few
+    kilobytes, however long the whole record is."""
+    import json
+    line = {"metric": bench.METRIC, "value": 1.0, "unit": "GFLOP/s", "n_gpus": 1, "steps": 5, "warmup": 3,
+            "ms_per_step": 1.0, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
+            "data": "synthetic", "config": {"workload": "w" * 300, "n": 16384}, "roofline": {"kernel": "gemm_tc"},
+            "e2e": {"value": 1.0, "unit": "GFLOP/s", "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 1},
+            "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": []}, "gpu_launches": 9,
+            "check": {"ok": True}, "lu_forms": {"fp64": {"ms": 1.0, "kernels": ["k"] * 1000}, "n": 16384},
+            "kernels": {f"k{i}": {"ms": 1.0} for i in range(1000)}, "serving": {"x": list(range(10000))}}
+    out = bench.headline(line)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "e2e", "clocks", "gpu_launches"):
+        assert out[k] == line[k]
+    assert out["lu_forms_ms"] == {"fp64": 1.0}
+    assert len(json.dumps(out)) < 4000
