@@ -15,7 +15,8 @@ _BINDING_NAMES = {
     "calu_factor_mixed", "ca_gesv_mixed_workspace", "calu_gesv_mixed", "ca_caqr_mixed_workspace",
     "caqr_factor_mixed", "ca_batched_plan", "ca_batched_factor", "BatchedFactor", "ca_batch_item_t",
     "CA_BATCH_CALU", "CA_BATCH_CAQR", "CA_DTYPE_F64", "CA_DTYPE_F32", "ca_solve_status",
-    "ca_getrs_workspace", "ca_test_solve_hook", "ca_test_cluster_hook", "ca_test_panel_hook", "CA_STATUS_PANEL_TIMEOUT", "CA_REFINE_CLASSIC", "CA_REFINE_GMRES", "CA_REFINE_AUTO",
+    "ca_getrs_workspace", "ca_test_solve_hook", "ca_test_cluster_hook", "ca_test_panel_hook",
+    "CA_STATUS_PANEL_TIMEOUT", "CA_REFINE_CLASSIC", "CA_REFINE_GMRES", "CA_REFINE_AUTO",
     "CA_STATUS_SOLVE_TIMEOUT", "CA_STATUS_REFACTORED", "ca_peak_probe", "ca_gels_mixed_workspace",
     "caqr_gels_mixed",
 }

@@ -94,6 +94,28 @@ def test_lu_keeps_weak_couplings(ca, b, delta):
     check(lu_err(to_host(F), LU_o), 1e-12, (b, delta))
 
 
+@pytest.mark.parametrize("m,n,b", [(190, 190, 64), (333, 421, 48), (421, 333, 32), (385, 513, 128), (300, 161, 128)])
+def test_lu_weak_couplings_in_some_blocks(ca, m, n, b):
+    """The first panel's unknowns numbered in turn, the others group by group:
+    only the blocks that join a group's rows to the other's columns hold
+    elements that the digits cannot stand for; ragged tiles on both sides."""
+    L, delta = 128, 1e-9
+    A = inputs.gaussian(m, n, m + n + b)
+    i, K = np.arange(max(m, n)), min(m, n)
+    group = np.where((i < b) | (i >= K), i % 2, i >= b + (K - b) // 2)   # as many rows as columns in each
+    row, col = group[:m], group[:n]
+    A = np.asfortranarray(np.where(row[:, None] == col[None, :], A, delta * A))
+    LU_o, ipiv_o, info_o, _ = oracle.calu(A, b, oracle.make_tree(L))
+    F = to_dev(A)
+    before = ca.ca_launch_count(9)
+    ipiv, info = ca.calu_factor(F, b, ca.make_tree(L))
+    torch.cuda.synchronize()
+    assert (ca.ca_launch_count(9) > before) == (K - b >= 64)
+    assert info.cpu().tolist() == [info_o, 0]
+    assert np.array_equal(ipiv.cpu().numpy(), ipiv_o)
+    check(lu_err(to_host(F), LU_o), 1e-12, (m, n, b))
+
+
 def qr_run(ca, A, b, tree, work=None):
     F = to_dev(A)
     before = ca.ca_launch_count(9)
