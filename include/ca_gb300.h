@@ -226,10 +226,10 @@ int calu_getrs(int n, int nrhs, const double *LU, int lda, const int *ipiv, doub
  *   2. the trailing columns get every leaf's Q^T (UPFACT), then every merge
  *      node's Q^T bottom-up (UPELIM); with the queried workspace large updates
  *      run on the tensor cores from exact digits, as in calu_factor, for the
- *      elements whose error is then at most ten times the bound of FP64
+ *      elements whose error is then at most eighty times the bound of FP64
  *      multiply-adds in the same product, and in FP64 for the others (the
- *      measured error is 0.8 to 1.5 times that of the FP64 pipe, for rows
- *      weighted by up to 2^40 too).
+ *      measured error of the factorization is 0.8 to 1.6 times that of the
+ *      FP64 pipe, for rows weighted by up to 2^40 too).
  * Q is kept in the compact Y T Y^T form (Sec. 3.1), stored in a tree
  * structure:
  *   - leaf j of panel k: Householder vectors strictly below the leaf-local

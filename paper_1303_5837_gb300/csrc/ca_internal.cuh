@@ -319,7 +319,9 @@ struct TcGemm {
   // in FP64 (tc_check_kernel).  kexp: A's column k is taken times 2^-kexp[k]
   // and B's row k times 2^kexp[k] (exact; null: 0).  reuse_a: A's digits of
   // the previous call with this workspace, A and kexp are still in place.
+  // czero: C is zero (the check need not read it).
   float keep;
+  int czero;
   const int *kexp;
   int reuse_a;
 };
@@ -344,7 +346,7 @@ size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, i
 cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, int leaf_rows, const Plan &plan,
                              const double *Tp, double *C, int ldc, int ncols, const QrPanelWs &ws, void *tcws,
                              int S, int exact, int *status, cudaStream_t st, float keep = 0.0f);
-constexpr float kTreeKeep = 1.0f / 32;  // TcGemm::keep of the FP64 tree update (update_tc.cu)
+constexpr float kTreeKeep = 1.0f / 256;  // TcGemm::keep of the FP64 tree update (update_tc.cu)
 // whether the FP64 update (7 exact digits, keep > 0) is faster there than on
 // the FP64 pipe
 bool tree_tc_pays(int mk, int bk, int ncols, int leaf_rows, const Plan &plan);

@@ -338,6 +338,7 @@ struct TcArgs {
   const int *skip;     // nonzero: a stage enqueued ahead that is not needed, do nothing
   int slices;          // operand slices per item: S digits, then the magnitudes when keep > 0
   float keep;          // TcGemm::keep
+  int czero;           // TcGemm::czero
   unsigned *fp64;      // keep > 0: bit c of word [item][row / 32][column / 32]: these 32 rows of column c take FP64
   TcOperand A, B;
 };
@@ -691,11 +692,12 @@ __global__ void __launch_bounds__(256, 2)
 // depends on nothing but those rows and that column: the result does not
 // change with the way a matrix is cut into calls.  Non-finite vectors and
 // those with values near the ends of the range (kExOdd) take it too.
-// Bound by its launch and the chain load - MMA - read for small updates, by the
-// operands' L2 reads for large ones: CALU + solve of n = 10240 113.4 -> 114.5
-// ms (no element fails there), CAQR + solve of n = 6144 128.2 -> 146.0 ms
-// (1335 checks of about 15 us; 6 % of the updates' blocks of 32 x 32 hold an
-// element that fails, mostly in T^T W, 2 % of their columns).
+// Bound by the chain load - MMA - read of a CTA, about 3 us: 2016 CTAs take 28
+// us where the digits' split takes 300 and their product 540 (16 leaves, K =
+// 128, 16128 columns); 127 us where most elements have to look at C.  The
+// first form compared in FP64 and took four times as long.  With the FP64
+// blocks: CALU + solve of n = 10240 113.3 -> 113.9 ms (no element fails),
+// CAQR + solve of n = 6144 128.3 -> 131.6, CAQR of n = 16384 887 -> 906.
 // --------------------------------------------------------------------------
 constexpr int kChkN = 128;
 
@@ -765,14 +767,36 @@ __global__ void __launch_bounds__(256, 3)
     const int myec = mycol < nvv ? a.eb[(size_t)item * a.npad + mycol] : 0;
     unsigned fail = __ballot_sync(0xffffffffu, myec > kExOdd / 2);
     if (er > kExOdd / 2 || !ok) fail = 0xffffffffu;
+    // FP32 and integers only: an FP64 instruction would hold the pipe for 64
+    // clocks, and most of them for nothing
+    unsigned low = 0;
 #pragma unroll
     for (int c = 0; c < 32; ++c) {
       const float v = __uint_as_float(r[c]);
-      const int ec = __shfl_sync(0xffffffffu, myec, c);
-      if (v < a.keep && v != 0.0f && !((fail >> c) & 1u)) {
-        // rin and the column is valid: padding has no magnitudes
-        const double lack = (double)(a.keep - v) * pow2i(er + ec);
-        if (er + ec > 1000 || !(fabs(Cb[row + (size_t)(n0 + c0 + c) * a.ldc]) >= lack)) fail |= 1u << c;
+      low |= (v < a.keep && v != 0.0f) ? 1u << c : 0u;
+    }
+    low = rin ? low & ~fail : 0u;  // (padding columns have no magnitudes)
+    if (a.czero) {  // no C to add
+      fail |= low;
+    } else if (__any_sync(0xffffffffu, low != 0u)) {
+      constexpr int kAt = 16;  // loads of C in flight
+#pragma unroll
+      for (int c1 = 0; c1 < 32; c1 += kAt) {
+        if (!__any_sync(0xffffffffu, (low >> c1 & 0xffffu) != 0u)) continue;
+        unsigned long long cb[kAt];
+#pragma unroll
+        for (int j = 0; j < kAt; ++j)
+          cb[j] = (low >> (c1 + j) & 1u) ? absbits(Cb[row + (size_t)(n0 + c0 + c1 + j) * a.ldc]) : 0ull;
+#pragma unroll
+        for (int j = 0; j < kAt; ++j) {
+          const int ec = __shfl_sync(0xffffffffu, myec, c1 + j);
+          // |C| 2^-(e_i + f_j) rounded down to a float's bits
+          const int E = (int)(cb[j] >> 52), ef = E - 1023 + 127 - er - ec;
+          const float f = E == 0 || ef <= 0 ? 0.0f
+                          : ef >= 254      ? 1e38f
+                                           : __uint_as_float(((unsigned)ef << 23) | (unsigned)(cb[j] >> 29 & 0x7fffffull));
+          if ((low >> (c1 + j) & 1u) && (E == 0x7ff || !(__uint_as_float(r[c1 + j]) + f >= a.keep))) fail |= 1u << (c1 + j);
+        }
       }
     }
     fail = __reduce_or_sync(0xffffffffu, rin ? fail : 0u);
@@ -803,7 +827,7 @@ struct SplitSide {
 };
 
 template <bool KEEP, int S>
-__global__ void __launch_bounds__(256) split_kernel(const __grid_constant__ SplitSide sideA,
+__global__ void __launch_bounds__(256, KEEP ? 4 : 1) split_kernel(const __grid_constant__ SplitSide sideA,
                                                     const __grid_constant__ SplitSide sideB, int nblkA, int nbatch,
                                                     int kpad, int exact, const int *skip, const int *kexp) {
   if (skip && *skip) return;
@@ -821,7 +845,7 @@ __global__ void __launch_bounds__(256) split_kernel(const __grid_constant__ Spli
   const int nv = o.nv_item ? o.nv_item[b] : (last ? o.nv_last : o.nv);
   const int K = operand_k(o, b, last);
   const double *X = operand_item(o, b);
-  constexpr int kPer = 8;  // K <= 256
+  constexpr int kPer = KEEP ? 4 : 8;  // K <= 128 (exact sums), 256
   constexpr int kSlices = S + (KEEP ? 1 : 0);
   double x[kPer];
   int sh[kPer];            // the element is taken times 2^sh
@@ -834,36 +858,39 @@ __global__ void __launch_bounds__(256) split_kernel(const __grid_constant__ Spli
     double val = 0.0;
     if (v < nv && k < K) val = operand_at(o, X, v, k);
     x[t] = val;
-    const unsigned long long bits = absbits(val);
-    mx = bits > mx ? bits : mx;
     sh[t] = 0;
     if constexpr (KEEP) {
+      const int E = (int)(__double2hiint(val) >> 20) & 0x7ff;
+      const bool some = absbits(val) != 0ull;
       if (kexp && k < K) sh[t] = ksign * kexp[k];
-      if (bits != 0) me = max(me, (int)(bits >> 52) + sh[t]);
-      odd |= (bits >> 52) == 0x7ffull || ((bits >> 52) == 0 && bits != 0);  // (the digits drop subnormals)
+      if (some) me = max(me, E + sh[t]);
+      odd |= some && (unsigned)(E - 1) >= 0x7feu;  // not finite, or subnormal (the digits drop those)
+    } else {
+      const unsigned long long bits = absbits(val);
+      mx = bits > mx ? bits : mx;
     }
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const unsigned long long ot = __shfl_xor_sync(0xffffffffu, mx, off);
-    mx = ot > mx ? ot : mx;
-  }
-  // |x| < 2^e; e from the exponent field of the largest magnitude
-  int e = 0;
-  if (mx != 0) {
-    const int E = (int)(mx >> 52);
-    e = (E == 0) ? -1021 : E - 1022;
-  }
+  int e = 0;  // |x| < 2^e, from the exponent field of the largest magnitude
   if constexpr (KEEP) {
     me = __reduce_max_sync(0xffffffffu, me);
     odd = __reduce_or_sync(0xffffffffu, odd);
-    if (mx != 0) {
+    if (me != INT_MIN) {
       e = me - 1022;
       if (odd || e < -900 || e > 1000) {  // no digits: FP64
         e = kExOdd;
 #pragma unroll
         for (int t = 0; t < kPer; ++t) x[t] = 0.0;
       }
+    }
+  } else {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long ot = __shfl_xor_sync(0xffffffffu, mx, off);
+      mx = ot > mx ? ot : mx;
+    }
+    if (mx != 0) {
+      const int E = (int)(mx >> 52);
+      e = (E == 0) ? -1021 : E - 1022;
     }
   }
   if (lane == 0) ex[(long long)b * vpad + v] = e;
@@ -889,11 +916,11 @@ __global__ void __launch_bounds__(256) split_kernel(const __grid_constant__ Spli
       out[(((long long)b * kSlices + s) * vpad + v) * kpad + k] = __float2bfloat16_rn(d * w);
     }
     if constexpr (KEEP) {
-      const unsigned long long bits = absbits(x[t]);
-      const int ed = (int)(bits >> 52) - 1023 + sh[t] - e;  // below 0; a subnormal's is not used
-      const unsigned m = bits == 0 ? 0u : ed < -40 || (bits >> 52) == 0 ? (127u - 40u) << 7
-                                                    : ((unsigned)(127 + ed) << 7) | (unsigned)((bits >> 45) & 0x7f);
-      out[(((long long)b * kSlices + S) * vpad + v) * kpad + k] = __ushort_as_bfloat16((unsigned short)m);
+      // exponent field and the first 7 bits of the mantissa, the exponent
+      // moved from the double's bias to the bfloat's and by sh - e
+      const int m = ((__double2hiint(x[t]) & 0x7fffffff) >> 13) + (sh[t] - e - (1023 - 127)) * 128;
+      const unsigned mag = absbits(x[t]) == 0ull ? 0u : (unsigned)max(m, (127 - 40) * 128);
+      out[(((long long)b * kSlices + S) * vpad + v) * kpad + k] = __ushort_as_bfloat16((unsigned short)mag);
     }
   }
 }
@@ -1098,6 +1125,7 @@ cudaError_t gemm_tc(const TcGemm &g, void *ws, int *status, cudaStream_t st) {
   a.skip = g.skip;
   a.slices = (int)ns;
   a.keep = g.keep;
+  a.czero = g.czero;
   a.fp64 = (unsigned *)p;
   a.A = g.A;
   a.B = g.B;

@@ -84,12 +84,16 @@ size_t tree_tc_ws_bytes(int mk, int bk, int ncols, int leaf_rows, int nleaves, i
 // The FP64 tree update from 7 digits.  As in the Schur update (gemm_tc.cu) an
 // element that is small beside its vectors' largest is multiplied in FP64, so
 // that heavy rows do not take the light ones' digits.  The line (kTreeKeep) is
-// a tenth of the Schur update's: sums of one or two terms (the top rows of a
-// leaf, the first reflectors of a merge) come near any line by chance, and at
-// 2.5 / 8 nearly every block that holds one would run in FP64.  An element's
-// error bound is therefore up to ten times that of FP64 multiply-adds; the
-// measured error of CAQR is 0.8 to 1.5 times that of the FP64 kernels (2000 x
-// 1400, the first rows weighted by 2^0 .. 2^40).  The update is a
+// an eightieth of the Schur update's.  Sums of one or two terms (the top rows
+// of a leaf, the first reflectors of a merge) come near any line by chance; and
+// what the sums over a leaf's rows lack of exact ones is relative to
+// |Y|^T |C|, not to what is left of W by chance, and goes on through T and Y.
+// At 1 / 32 every block that holds such a row had an element to multiply (6 %
+// of all blocks; CAQR of n = 16384 1072 ms, 906 now); without any line the
+// error matches the FP64 kernels' up to weights of 2^12 (2000 x 1400, the
+// first rows weighted: 2.0e-14 against 1.3e-14 at 2^8, 1.4e-13 against 1.1e-13
+// at 2^12, 8.0e-12 against 1.6e-13 at 2^20), with it for all weights to 2^40
+// (0.8 to 1.6 times).  The update is a
 // chain of many small launches (split, check and product per contraction of up
 // to 128 rows), so it pays where the FP64 kernels would take longer than some
 // time per launch at the 0.5 TFLOP/s they reach on the shapes near the line
@@ -208,6 +212,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
     g2.S = S;
     g2.exact = exact;
     g2.keep = keep;
+    g2.czero = 1;
     if ((e = gemm_tc(g2, gws, status, st)) != cudaSuccess) return e;
     // C -= Y W'
     TcGemm g3 = {};
@@ -309,6 +314,7 @@ cudaError_t tree_apply_qt_tc(int mk, int bk, int b, const double *P, int lda, in
       g2.S = S;
       g2.exact = exact;
       g2.keep = keep;
+      g2.czero = 1;
       if ((e = gemm_tc(g2, gws, status, st)) != cudaSuccess) return e;
       {
         ProfScope ps(kClsTreeApply, st, 0.0);

@@ -132,8 +132,7 @@ def test_qr_keeps_light_rows_below_heavy_ones(ca, w, b, L, lv):
     weights), so that the first panel has heavy reflectors and light ones: the
     rows of R below them are those of the light part.  Their distance from the
     oracle, columnwise, is at most 11 times that of the same factorization on
-    the FP64 pipe: the line of the digit form bounds its errors by ten times
-    the bound of multiply-adds, and the oracle's own error is in both."""
+    the FP64 pipe (ten times its error, and the oracle's own is in both)."""
     m, n = 2000, 1400
     A = inputs.gaussian(m, n, 31 + b)
     h = b // 2
