@@ -827,9 +827,9 @@ struct SplitSide {
 };
 
 template <bool KEEP, int S>
-__global__ void __launch_bounds__(256, KEEP ? 4 : 1) split_kernel(const __grid_constant__ SplitSide sideA,
-                                                    const __grid_constant__ SplitSide sideB, int nblkA, int nbatch,
-                                                    int kpad, int exact, const int *skip, const int *kexp) {
+__global__ void __launch_bounds__(256, KEEP ? 4 : 1)
+    split_kernel(const __grid_constant__ SplitSide sideA, const __grid_constant__ SplitSide sideB, int nblkA, int nbatch,
+                 int kpad, int exact, const int *skip, const int *kexp) {
   if (skip && *skip) return;
   const bool second = (int)blockIdx.x >= nblkA;
   const SplitSide &d = second ? sideB : sideA;
